@@ -61,3 +61,40 @@ def test_bad_k(gb):
     with pytest.raises(gb.Fp8Error) as e:
         gb.prune24_compress(torch.zeros((2, 6), dtype=torch.uint8, device="cuda"))
     assert e.value.status == -2
+
+
+@pytest.mark.parametrize("M,K,pad", [(1, 16, 0), (3, 16, 0), (1025, 16, 0), (7, 1024, 0), (5, 1040, 16),
+                                     (2, 16400, 0), (33, 4096, 32), (6, 24, 0), (6, 24, 8), (4, 1028, 0)])
+def test_contiguous_and_strided_rows(orc, M, K, pad):
+    """Rows as one run of 16-code pieces (lda == K), row by row (padded
+    rows) and the scalar path (K % 16 != 0), at the edges of a block's 1024
+    pieces; the expansion of each on its vector and scalar paths."""
+    import paper_2602_10262_gb300 as gb
+    a = workloads.random_codes((M, K), seed=11 + M)
+    t = torch.zeros((M, K + pad), dtype=torch.uint8, device="cuda")
+    t[:, :K] = torch.from_numpy(a).cuda()
+    vals, meta = gb.prune24_compress(t[:, :K])
+    vo, mo = orc.prune24(a)
+    assert np.array_equal(vals.cpu().numpy(), vo) and np.array_equal(meta.cpu().numpy(), mo)
+    out = gb.prune24_decompress(vals, meta, K)
+    assert np.array_equal(out.cpu().numpy(), orc.decompress24(vo, mo, K))
+    # an output that starts off a 16-byte boundary takes the scalar path
+    buf = torch.zeros(M * K + 4, dtype=torch.uint8, device="cuda")
+    off = buf[4:].reshape(M, K)
+    gb.prune24_decompress(vals, meta, K, out=off)
+    assert torch.equal(off, out)
+
+
+def test_expand_any_index_nibble(orc):
+    """Metadata is the caller's: equal or descending indices expand the same
+    on the vector and the scalar path."""
+    import paper_2602_10262_gb300 as gb
+    M, K = 4, 512
+    g = torch.Generator().manual_seed(3)
+    vals = torch.randint(0, 256, (M, K // 2), generator=g, dtype=torch.int32).to(torch.uint8).cuda()
+    meta = torch.randint(0, 256, (M, K // 8), generator=g, dtype=torch.int32).to(torch.uint8).cuda()
+    out = gb.prune24_decompress(vals, meta, K)
+    buf = torch.zeros(M * K + 4, dtype=torch.uint8, device="cuda")
+    off = buf[4:].reshape(M, K)
+    gb.prune24_decompress(vals, meta, K, out=off)
+    assert torch.equal(off, out)
