@@ -1,11 +1,12 @@
 // Scale selection + FP8 quantisation (fp8_quantize_e4m3, fp8_quantize_e5m2).
 //
-// Per row (scale_mode 1): one CTA per row.  Pass 1 takes amax of the row with
-// 16-byte loads and a warp/CTA max reduction on the fp32 bit patterns of |x|
-// (monotone for non-negative floats; Inf and NaN compare above every finite
-// value, which is how non-finite input is detected).  Pass 2 re-reads the
-// row (an L2 hit: the rows in flight are far smaller than L2) and writes the
-// codes.  HBM traffic: 4 bytes read + 1 byte written per element.
+// Per row (scale_mode 1): a group of TPR threads holds a whole row in
+// registers: it is loaded once, its amax is a max reduction on the fp32 bit
+// patterns of |x| (monotone for non-negative floats; Inf and NaN compare
+// above every finite value, which is how non-finite input is detected), and
+// the codes come from the registers.  Rows of more than kRowMaxCols columns
+// are read twice instead, the second time from L2.  HBM traffic: 4 bytes
+// read + 1 byte written per element.
 //
 // fp8_quantize_e4m3_rows_grouped runs the per-row path for up to 32
 // independent matrices in one launch (job table in the kernel parameters).
@@ -18,6 +19,8 @@
 // format's largest finite value (448 for E4M3, 57344 for E5M2), and each code
 // is cvt.rn.satfinite of the IEEE product x * s (__fmul_rn) to that format.
 // Every kernel is a template on the format (FMT 0: E4M3, 1: E5M2).
+#include <algorithm>
+
 #include <cuda_fp8.h>
 
 #include "common.cuh"
@@ -90,8 +93,257 @@ __device__ __forceinline__ void scale_from_amax(uint32_t amax_bits, float& s, fl
     }
 }
 
-// One row: amax (CTA reduction), scale, codes.  vec: the row allows 16-byte
-// loads and 4-byte stores (x 16-aligned, q 4-aligned).
+// ---------------------------------------------------------------- rows in registers
+//
+// TPR threads (a warp, or a whole number of warps of one block) take a row,
+// each holding U vectors of W consecutive elements: vector u of thread t
+// starts at column (u * TPR + t) * W.  W = 8 is one 32-byte load a vector
+// (x 32-aligned, ldx % 8 == 0), W = 4 one 16-byte load, or guarded scalar
+// loads where x allows neither and past the last whole vector.
+//
+// What bounds it: HBM, once enough bytes are in flight.  Rows are loaded
+// once instead of twice (the second pass over L2 cost issue slots and load
+// latency with nothing else to do), short rows share a block (one warp each
+// up to 1024 columns) and the few long rows of a decode step get up to 1024
+// threads each, since there the row's own latency is all there is.
+// Measured (GB300, inputs rotated beyond L2), against one block of 256
+// threads per row that read it twice: 16384 x 4096 58.0 -> 49.2 us (6.8
+// TB/s), 16384 x 14336 183 -> 165 us (7.1 TB/s), 16384 x 512 28.5 -> 8.5 us,
+// 16 x 14336 3.4 -> 2.5 us.  Fused with 2:4 compression: 14336 x 4096 64.7
+// -> 50.2 us (6.6 TB/s), 16384 x 16384 250 -> 216 us (its ALU pipe was 68 %
+// busy: the four-group selection took half of that away).
+constexpr int kRowBlock = 256;            // threads of a block where TPR is smaller
+constexpr int kRowMaxCols = 16384;        // longest row held in registers
+
+template <int TPR>
+constexpr int row_block()
+{
+    return TPR > kRowBlock ? TPR : kRowBlock;
+}
+
+// W consecutive floats at p, the first `left` of them inside the row (0 for
+// the others).  vec: p is aligned for whole-vector loads.
+template <int W>
+__device__ __forceinline__ void load_vec(const float* p, int64_t left, bool vec, float (&v)[W])
+{
+    if (vec && left >= W) {
+        if constexpr (W == 8) {
+            asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+                           "=f"(v[7])
+                         : "l"(p));
+        } else {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+            v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            v[i] = i < left ? __ldg(p + i) : 0.0f;
+    }
+}
+
+// As load_vec<8> for rows that are only 16-byte aligned (left is 0 or >= 8).
+__device__ __forceinline__ void load_two_vec4(const float* p, int64_t left, float (&v)[8])
+{
+    const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 a = left > 0 ? __ldg(reinterpret_cast<const float4*>(p)) : z;
+    const float4 b = left > 0 ? __ldg(reinterpret_cast<const float4*>(p) + 1) : z;
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+}
+
+// Max over the TPR threads of a row group.  red: one entry per warp of the
+// block, not in use by an earlier call since the last barrier.
+template <int TPR>
+__device__ __forceinline__ uint32_t row_max(uint32_t m, uint32_t* red)
+{
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if constexpr (TPR > 32) {
+        constexpr int kWarps = TPR / 32;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (lane == 0)
+            red[warp] = m;
+        __syncthreads();
+        const int first = warp / kWarps * kWarps;
+        m = __reduce_max_sync(0xFFFFFFFFu, lane < kWarps ? red[first + lane] : 0u);
+    }
+    return m;
+}
+
+template <int U, int W>
+__device__ __forceinline__ uint32_t held_amax(const float (&v)[U][W])
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            m = max(m, abs_bits(v[u][i]));
+    return m;
+}
+
+template <int FMT>
+__device__ __forceinline__ uint32_t enc4(const float* v, float s)
+{
+    return enc4<FMT>(make_float4(v[0], v[1], v[2], v[3]), s);
+}
+
+// The codes of one vector to qr (qa: the row's store alignment, 8, 4 or 1).
+template <int FMT, int W>
+__device__ __forceinline__ void store_codes(uint8_t* qr, int64_t left, int qa, const float (&v)[W], float s)
+{
+    if (left <= 0)
+        return;
+    uint32_t w[W / 4];
+#pragma unroll
+    for (int h = 0; h < W / 4; ++h)
+        w[h] = enc4<FMT>(v + 4 * h, s);
+    if (left >= W && qa >= W) {
+        if constexpr (W == 8)
+            *reinterpret_cast<uint2*>(qr) = make_uint2(w[0], w[1]);
+        else
+            *reinterpret_cast<uint32_t*>(qr) = w[0];
+    } else if (left >= W && qa >= 4) {
+#pragma unroll
+        for (int h = 0; h < W / 4; ++h)
+            reinterpret_cast<uint32_t*>(qr)[h] = w[h];
+    } else {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (i < left)
+                qr[i] = static_cast<uint8_t>(w[i / 4] >> (8 * (i % 4)));
+    }
+}
+
+// One row by its TPR threads (t: index within them; ok: the row exists).
+template <int FMT, int TPR, int U, int W>
+__device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols, uint8_t* qr, float* d_out, bool vec,
+                                                  int qa, int* err, uint32_t* red, int t, bool ok)
+{
+    float v[U][W];
+    const int64_t n = ok ? cols : 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+        load_vec<W>(xr + c, n - c, vec, v[u]);
+    }
+    const uint32_t m = row_max<TPR>(held_amax(v), red);
+    float s, dq;
+    scale_from_amax<FMT>(m, s, dq);
+    if (t == 0 && ok) {
+        if (m >= kInfBits)
+            report_device_error(err, FP8_ERR_NONFINITE);
+        *d_out = dq;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+        store_codes<FMT, W>(qr + c, n - c, qa, v[u], s);
+    }
+}
+
+template <int FMT, int TPR, int U, int W>
+__global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float* __restrict__ x, int64_t rows,
+                                                                     int64_t cols, int64_t ldx,
+                                                                     uint8_t* __restrict__ q, int64_t ldq,
+                                                                     float* __restrict__ d, int vec, int qa, int* err)
+{
+    grid_launch_dependents();
+    __shared__ uint32_t red[2][32];
+    constexpr int kRows = row_block<TPR>() / TPR;         // rows per block
+    const int t = threadIdx.x % TPR;
+    int flip = 0;
+    for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRows; r0 < rows;
+         r0 += static_cast<int64_t>(gridDim.x) * kRows, flip ^= 1) {
+        const int64_t r = r0 + threadIdx.x / TPR;
+        quantize_held_row<FMT, TPR, U, W>(x + r * ldx, cols, q + r * ldq, d + r, vec != 0, qa, err, red[flip], t,
+                                          r < rows);
+    }
+}
+
+// Per-row E4M3 quantisation and 2:4 compression of the codes in one pass
+// (fp8_quantize_e4m3_prune24): as quant_row_kernel with W = 8, and a
+// thread's vectors two at a time are four 2:4 groups, whose kept codes and
+// index nibbles come from their codes exactly as prune24_compress's do
+// (select_groups4): 4 bytes of kept codes and one metadata byte per vector,
+// next to the neighbouring lanes'.  Needs cols % 128 == 0, x 16-aligned with
+// ldx % 4 == 0, q 4-aligned with ldq % 4 == 0, a_vals 2-aligned (checked by
+// the host).  wide: x rows are 32-aligned; out8: q rows are 8-aligned and
+// vals rows 4-aligned.
+template <int TPR, int U>
+__global__ void __launch_bounds__(row_block<TPR>()) quant_row_prune_kernel(const float* __restrict__ x, int64_t rows,
+                                                                           int64_t cols, int64_t ldx,
+                                                                           uint8_t* __restrict__ q, int64_t ldq,
+                                                                           float* __restrict__ d,
+                                                                           uint8_t* __restrict__ vals,
+                                                                           uint8_t* __restrict__ meta, int wide,
+                                                                           int out8, int* err)
+{
+    grid_launch_dependents();
+    __shared__ uint32_t red[2][32];
+    constexpr int kRows = row_block<TPR>() / TPR;
+    const int t = threadIdx.x % TPR;
+    const int64_t ldv = cols / 2, ldm = cols / 8;
+    int flip = 0;
+    for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRows; r0 < rows;
+         r0 += static_cast<int64_t>(gridDim.x) * kRows, flip ^= 1) {
+        const int64_t r = r0 + threadIdx.x / TPR;
+        const int64_t n = r < rows ? cols : 0;
+        const float* xr = x + r * ldx;
+        float v[U][8];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t c = static_cast<int64_t>(u * TPR + t) * 8;
+            if (wide)
+                load_vec<8>(xr + c, n - c, true, v[u]);
+            else
+                load_two_vec4(xr + c, n - c, v[u]);
+        }
+        const uint32_t m = row_max<TPR>(held_amax(v), red[flip]);
+        float s, dq;
+        scale_from_amax<0>(m, s, dq);
+        if (t == 0 && r < rows) {
+            if (m >= kInfBits)
+                report_device_error(err, FP8_ERR_NONFINITE);
+            d[r] = dq;
+        }
+        uint8_t* qr = q + r * ldq;
+        uint8_t* vr = vals + r * ldv;
+        uint8_t* mr = meta + r * ldm;
+        const auto put = [&](int64_t c, uint32_t w0, uint32_t w1, uint32_t kept, uint32_t nibs) {
+            if (c >= n)
+                return;
+            if (out8) {
+                *reinterpret_cast<uint2*>(qr + c) = make_uint2(w0, w1);
+                *reinterpret_cast<uint32_t*>(vr + c / 2) = kept;
+            } else {
+                reinterpret_cast<uint32_t*>(qr + c)[0] = w0;
+                reinterpret_cast<uint32_t*>(qr + c)[1] = w1;
+                reinterpret_cast<uint16_t*>(vr + c / 2)[0] = static_cast<uint16_t>(kept);
+                reinterpret_cast<uint16_t*>(vr + c / 2)[1] = static_cast<uint16_t>(kept >> 16);
+            }
+            mr[c / 8] = static_cast<uint8_t>(nibs);
+        };
+#pragma unroll
+        for (int u = 0; u < U; u += 2) {
+            const bool two = u + 1 < U;
+            const int u1 = two ? u + 1 : u;
+            const uint32_t w0 = enc4<0>(v[u], s), w1 = enc4<0>(v[u] + 4, s);
+            const uint32_t w2 = two ? enc4<0>(v[u1], s) : 0u, w3 = two ? enc4<0>(v[u1] + 4, s) : 0u;
+            uint32_t v01, v23;
+            const uint32_t nibs = select_groups4(w0, w1, w2, w3, &v01, &v23);
+            put(static_cast<int64_t>(u * TPR + t) * 8, w0, w1, v01, nibs);
+            if (two)
+                put(static_cast<int64_t>(u1 * TPR + t) * 8, w2, w3, v23, nibs >> 8);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- rows read twice
+
+// One row by a whole block of kThreads: amax, scale, codes.  vec: the row
+// allows 16-byte loads and 4-byte stores (x 16-aligned, q 4-aligned).
 template <int FMT>
 __device__ __forceinline__ void quantize_row(const float* __restrict__ xr, int64_t cols,
                                              uint8_t* __restrict__ qr, float* __restrict__ d_out,
@@ -120,14 +372,12 @@ __device__ __forceinline__ void quantize_row(const float* __restrict__ xr, int64
         qr[c] = static_cast<uint8_t>(enc2<FMT>(__fmul_rn(xr[c], s), 0.0f) & 0xFFu);
 }
 
-// vec: x rows and q rows allow 16-byte loads / 4-byte stores (x 16-aligned,
-// ldx % 4 == 0, q 4-aligned, ldq % 4 == 0).
 template <int FMT>
-__global__ void __launch_bounds__(kThreads) quant_row_kernel(const float* __restrict__ x,
-                                                             int64_t rows, int64_t cols,
-                                                             int64_t ldx, uint8_t* __restrict__ q,
-                                                             int64_t ldq, float* __restrict__ d,
-                                                             int vec, int* err)
+__global__ void __launch_bounds__(kThreads) quant_long_row_kernel(const float* __restrict__ x,
+                                                                  int64_t rows, int64_t cols,
+                                                                  int64_t ldx, uint8_t* __restrict__ q,
+                                                                  int64_t ldq, float* __restrict__ d,
+                                                                  int vec, int* err)
 {
     grid_launch_dependents();
     __shared__ uint32_t red[kThreads / 32];
@@ -135,26 +385,15 @@ __global__ void __launch_bounds__(kThreads) quant_row_kernel(const float* __rest
         quantize_row<FMT>(x + r * ldx, cols, q + r * ldq, d + r, vec, err, red);
 }
 
-// Per-row E4M3 quantisation and 2:4 compression of the codes in one pass
-// (fp8_quantize_e4m3_prune24).  Pass 1 takes the row's amax as quantize_row
-// does; pass 2 re-reads the row (from L2) and encodes four elements (one 2:4
-// group) per lane and step, with coalesced 16-byte loads and 4-byte code
-// stores, and selects the group's two kept codes and index nibble from its
-// codes exactly as prune24_compress does (prune_select.cuh); lanes 2i and
-// 2i + 1 hold consecutive groups and combine their nibbles into one
-// metadata byte.  Measured against fp8_quantize_e4m3 followed by
-// prune24_compress: 252 against 275 us at 16384 x 16384, 68 against 79 us
-// at 8192 x 8192.  Staging each row in shared memory (no second read from
-// L2 or DRAM, but three CTAs per SM at 16384 columns) and persistent grids
-// of four or eight CTAs per SM were slower.  Needs cols % 128 == 0 (so
-// every warp runs the same number of steps), x 16-aligned with ldx % 4 ==
-// 0, q 4-aligned with ldq % 4 == 0, a_vals 2-aligned (checked by the host).
-__global__ void __launch_bounds__(kThreads) quant_row_prune_kernel(const float* __restrict__ x, int64_t rows,
-                                                                   int64_t cols, int64_t ldx,
-                                                                   uint8_t* __restrict__ q, int64_t ldq,
-                                                                   float* __restrict__ d,
-                                                                   uint8_t* __restrict__ vals,
-                                                                   uint8_t* __restrict__ meta, int* err)
+// Rows of more than kRowMaxCols columns, quantised and compressed: the
+// encode pass re-reads the row and takes one 2:4 group per lane and step
+// (lanes 2i and 2i + 1 join their nibbles into one metadata byte).
+__global__ void __launch_bounds__(kThreads) quant_long_row_prune_kernel(const float* __restrict__ x, int64_t rows,
+                                                                        int64_t cols, int64_t ldx,
+                                                                        uint8_t* __restrict__ q, int64_t ldq,
+                                                                        float* __restrict__ d,
+                                                                        uint8_t* __restrict__ vals,
+                                                                        uint8_t* __restrict__ meta, int* err)
 {
     grid_launch_dependents();
     __shared__ uint32_t red[kThreads / 32];
@@ -193,28 +432,55 @@ __global__ void __launch_bounds__(kThreads) quant_row_prune_kernel(const float* 
 
 // Many independent per-row quantisations in one launch: the job table is
 // passed by value; CTA b takes global row b (rows of job j follow those of
-// job j - 1).
+// job j - 1), held in the registers of kGroupedTpr threads (U: enough for
+// the longest row), or read twice where a row is longer than that allows.
 struct RowJobs {
     fp8_quant_job job[FP8_QUANT_GROUPED_MAX];
     int64_t row_start[FP8_QUANT_GROUPED_MAX + 1];
-    int vec[FP8_QUANT_GROUPED_MAX];
+    int vec[FP8_QUANT_GROUPED_MAX];       // whole-vector loads of the launch's W (or, read twice, of 4)
+    int qa[FP8_QUANT_GROUPED_MAX];        // store alignment of the codes: 8, 4 or 1
     int n;
 };
 
-__global__ void __launch_bounds__(kThreads) quant_rows_grouped_kernel(const __grid_constant__ RowJobs jobs,
-                                                                      int* err)
+constexpr int kGroupedTpr = 512;
+
+__device__ __forceinline__ int job_of_row(const RowJobs& jobs, int64_t g)
+{
+    int j = 0;
+    while (j + 1 < jobs.n && jobs.row_start[j + 1] <= g)
+        ++j;
+    return j;
+}
+
+template <int U, int W>
+__global__ void __launch_bounds__(kGroupedTpr) quant_rows_grouped_kernel(const __grid_constant__ RowJobs jobs,
+                                                                         int* err)
+{
+    grid_launch_dependents();
+    __shared__ uint32_t red[2][32];
+    const int64_t total = jobs.row_start[jobs.n];
+    int flip = 0;
+    for (int64_t g = blockIdx.x; g < total; g += gridDim.x, flip ^= 1) {
+        const int j = job_of_row(jobs, g);
+        const fp8_quant_job& J = jobs.job[j];
+        const int64_t r = g - jobs.row_start[j];
+        quantize_held_row<0, kGroupedTpr, U, W>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r,
+                                                jobs.vec[j] != 0, jobs.qa[j], err, red[flip], threadIdx.x, true);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) quant_long_rows_grouped_kernel(const __grid_constant__ RowJobs jobs,
+                                                                           int* err)
 {
     grid_launch_dependents();
     __shared__ uint32_t red[kThreads / 32];
     const int64_t total = jobs.row_start[jobs.n];
     for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
-        int j = 0;
-        while (j + 1 < jobs.n && jobs.row_start[j + 1] <= g)
-            ++j;
+        const int j = job_of_row(jobs, g);
         const fp8_quant_job& J = jobs.job[j];
         const int64_t r = g - jobs.row_start[j];
-        quantize_row<0>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r, jobs.vec[j], err,
-                     red);
+        quantize_row<0>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r, jobs.vec[j] && jobs.qa[j] >= 4,
+                        err, red);
     }
 }
 
@@ -283,6 +549,103 @@ __global__ void quant_finalize_kernel(uint32_t* slot, int* err)
     *reinterpret_cast<float*>(slot) = dq;
 }
 
+// Alignment of matrix rows of `esz`-byte elements: the largest of 8, 4 and
+// 1 elements that every row starts on a multiple of.
+int row_align(const void* p, int64_t ld, int esz)
+{
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    if (a % (8 * esz) == 0 && ld % 8 == 0)
+        return 8;
+    return a % (4 * esz) == 0 && ld % 4 == 0 ? 4 : 1;
+}
+
+int row_grid(int64_t rows, int rows_per_block)
+{
+    const int64_t blocks = (rows + rows_per_block - 1) / rows_per_block;
+    return static_cast<int>(std::min<int64_t>(blocks, 65535LL * 8));
+}
+
+// Calls f.template operator()<TPR, U8>() with the threads per row and
+// 8-element vectors per thread for rows of `cols` columns.  Few rows (no
+// more than two per SM): as many threads as the row has work for.  Many:
+// warps up to 1024 columns, then blocks of 128 to 512 threads with two to
+// four vectors each, in steps of a vector where half a vector more would
+// leave lanes idle (4100 columns: 16.5 us for 4096 rows with three vectors
+// a thread, 20.8 with four).
+template <typename F>
+void with_row_shape(int64_t rows, int64_t cols, F f)
+{
+    if (rows <= 2 * sm_count()) {
+        if (cols <= 1024)
+            f.template operator()<128, 1>();
+        else if (cols <= 4096)
+            f.template operator()<512, 1>();
+        else
+            f.template operator()<1024, 2>();
+    } else if (cols <= 256) {
+        f.template operator()<32, 1>();
+    } else if (cols <= 512) {
+        f.template operator()<32, 2>();
+    } else if (cols <= 1024) {
+        f.template operator()<32, 4>();
+    } else if (cols <= 2048) {
+        f.template operator()<128, 2>();
+    } else if (cols <= 4096) {
+        f.template operator()<256, 2>();
+    } else if (cols <= 6144) {
+        f.template operator()<256, 3>();
+    } else if (cols <= 8192) {
+        f.template operator()<256, 4>();
+    } else if (cols <= 12288) {
+        f.template operator()<512, 3>();
+    } else {
+        f.template operator()<512, 4>();
+    }
+}
+
+template <int FMT>
+struct RowLaunch {
+    const float* x;
+    int64_t rows, cols, ldx;
+    uint8_t* q;
+    int64_t ldq;
+    float* d;
+    int* err;
+    cudaStream_t st;
+
+    template <int TPR, int U>
+    void operator()() const
+    {
+        const int xa = row_align(x, ldx, 4), qa = row_align(q, ldq, 1);
+        const int grid = row_grid(rows, row_block<TPR>() / TPR);
+        if (xa == 8)
+            quant_row_kernel<FMT, TPR, U, 8><<<grid, row_block<TPR>(), 0, st>>>(x, rows, cols, ldx, q, ldq, d, 1, qa,
+                                                                                err);
+        else
+            quant_row_kernel<FMT, TPR, 2 * U, 4><<<grid, row_block<TPR>(), 0, st>>>(x, rows, cols, ldx, q, ldq, d,
+                                                                                    xa == 4, qa, err);
+    }
+};
+
+struct RowPruneLaunch {
+    const float* x;
+    int64_t rows, cols, ldx;
+    uint8_t* q;
+    int64_t ldq;
+    float* d;
+    uint8_t *vals, *meta;
+    int* err;
+    cudaStream_t st;
+
+    template <int TPR, int U>
+    void operator()() const
+    {
+        const int out8 = row_align(q, ldq, 1) == 8 && reinterpret_cast<uintptr_t>(vals) % 4 == 0;
+        quant_row_prune_kernel<TPR, U><<<row_grid(rows, row_block<TPR>() / TPR), row_block<TPR>(), 0, st>>>(
+            x, rows, cols, ldx, q, ldq, d, vals, meta, row_align(x, ldx, 4) == 8, out8, err);
+    }
+};
+
 template <int FMT>
 int quantize(const float* x, int64_t rows, int64_t cols, int64_t ldx, int scale_mode, uint8_t* q,
              int64_t ldq, float* dequant_scale, cudaStream_t st)
@@ -304,9 +667,11 @@ int quantize(const float* x, int64_t rows, int64_t cols, int64_t ldx, int scale_
                     (reinterpret_cast<uintptr_t>(q) % 4 == 0) && (ldq % 4 == 0);
     const int sms = sm_count();
     if (scale_mode == 1) {
-        const int64_t grid = rows < 65535LL * 8 ? rows : 65535LL * 8;
-        quant_row_kernel<FMT><<<static_cast<unsigned>(grid), kThreads, 0, st>>>(
-            x, rows, cols, ldx, q, ldq, dequant_scale, vec, err);
+        if (cols <= kRowMaxCols)
+            with_row_shape(rows, cols, RowLaunch<FMT>{x, rows, cols, ldx, q, ldq, dequant_scale, err, st});
+        else
+            quant_long_row_kernel<FMT><<<row_grid(rows, 1), kThreads, 0, st>>>(x, rows, cols, ldx, q, ldq,
+                                                                               dequant_scale, vec, err);
         GB_CUDA_OK(cudaGetLastError());
         return FP8_OK;
     }
@@ -593,9 +958,13 @@ extern "C" int fp8_quantize_e4m3_prune24(const float* x, int64_t rows, int64_t c
         return FP8_ERR_ALIGN;
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
-    const int64_t grid = rows < 65535LL * 8 ? rows : 65535LL * 8;
-    quant_row_prune_kernel<<<static_cast<unsigned>(grid), kThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-        x, rows, cols, ldx, q, ldq, dequant_scale, a_vals, a_meta, device_error_word());
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    int* err = device_error_word();
+    if (cols <= kRowMaxCols)
+        with_row_shape(rows, cols, RowPruneLaunch{x, rows, cols, ldx, q, ldq, dequant_scale, a_vals, a_meta, err, st});
+    else
+        quant_long_row_prune_kernel<<<row_grid(rows, 1), kThreads, 0, st>>>(x, rows, cols, ldx, q, ldq, dequant_scale,
+                                                                            a_vals, a_meta, err);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }
@@ -618,7 +987,8 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
         return FP8_ERR_SHAPE;
     RowJobs rj;
     memset(&rj, 0, sizeof(rj));
-    int64_t rows = 0;
+    int64_t rows = 0, max_cols = 0;
+    bool wide = true;
     for (int i = 0; i < num_jobs; ++i) {
         const fp8_quant_job& J = jobs[i];
         if (J.rows < 0 || J.cols < 0)
@@ -635,8 +1005,10 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
         const int k = rj.n++;
         rj.job[k] = J;
         rj.row_start[k] = rows;
-        rj.vec[k] = aligned16(J.x) && (J.ldx % 4 == 0) &&
-                    (reinterpret_cast<uintptr_t>(J.q) % 4 == 0) && (J.ldq % 4 == 0);
+        rj.vec[k] = row_align(J.x, J.ldx, 4);
+        rj.qa[k] = row_align(J.q, J.ldq, 1);
+        wide = wide && rj.vec[k] == 8;
+        max_cols = std::max(max_cols, J.cols);
         rows += J.rows;
     }
     rj.row_start[rj.n] = rows;
@@ -644,9 +1016,25 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
         return FP8_OK;
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
-    const int64_t grid = rows < 65535LL * 8 ? rows : 65535LL * 8;
-    quant_rows_grouped_kernel<<<static_cast<unsigned>(grid), kThreads, 0,
-                                reinterpret_cast<cudaStream_t>(stream)>>>(rj, device_error_word());
+    for (int i = 0; i < rj.n; ++i)
+        rj.vec[i] = rj.vec[i] >= 4;               // a row of the launch's W (wide: all 8) or of 4
+    const int grid = row_grid(rows, 1);
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    int* err = device_error_word();
+    const auto launch = [&](auto* w8, auto* w4) {
+        if (wide)
+            w8<<<grid, kGroupedTpr, 0, st>>>(rj, err);
+        else
+            w4<<<grid, kGroupedTpr, 0, st>>>(rj, err);
+    };
+    if (max_cols <= 8 * kGroupedTpr)
+        launch(quant_rows_grouped_kernel<1, 8>, quant_rows_grouped_kernel<2, 4>);
+    else if (max_cols <= 16 * kGroupedTpr)
+        launch(quant_rows_grouped_kernel<2, 8>, quant_rows_grouped_kernel<4, 4>);
+    else if (max_cols <= 32 * kGroupedTpr)
+        launch(quant_rows_grouped_kernel<4, 8>, quant_rows_grouped_kernel<8, 4>);
+    else
+        quant_long_rows_grouped_kernel<<<grid, kThreads, 0, st>>>(rj, err);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }

@@ -96,3 +96,57 @@ def test_device_encoder_all_in_range_fp32(gb, orc):
             got = q[:-1].reshape(-1)[:n].cpu().numpy()
             ref = orc.encode_pattern_range(lo | sign, (hi - 1 | sign) + 1)
             assert np.array_equal(got, ref), f"chunk at {lo | sign:#x}"
+
+
+# every threads-per-row / vectors-per-thread shape at its first and last
+# column counts, few rows and many (the rule counts rows per SM), and rows
+# longer than registers hold; each row stride and start: 32-byte, 16-byte
+# and no alignment of x, 8-, 4- and 1-byte alignment of the codes
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(r, c) for r in (9, 401) for c in
+                                       (1, 31, 256, 257, 512, 513, 1024, 1025, 2048, 2049, 4096, 4097, 6144, 6145,
+                                        8192, 8199, 12288, 12289, 16384, 16385)])
+def test_row_shapes(gb, orc, fmt, rows, cols):
+    x = workloads.randn_f32((rows, cols), seed=rows + cols)
+    x[rows // 2] = 0.0
+    x[0, cols - 1] = -1e4                                  # the row's amax in its last element
+    qo, do = orc.quantize(x, 1, fmt=fmt)
+    quantize = gb.fp8_quantize_e5m2 if fmt else gb.fp8_quantize_e4m3
+    for pad, off, qpad, qoff in ((-cols % 8, 0, -cols % 8, 0), (-cols % 4 + 4, 4, -cols % 4 + 4, 4), (1, 1, 1, 1)):
+        xb = torch.full((rows * (cols + pad) + off,), float("nan"), device="cuda")
+        xt = xb[off:].view(rows, cols + pad)[:, :cols]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((rows * (cols + qpad) + qoff,), 0xA5, dtype=torch.uint8, device="cuda")
+        qt = qb[qoff:].view(rows, cols + qpad)[:, :cols]
+        _, d = quantize(xt, 1, q=qt)
+        assert np.array_equal(d.cpu().numpy(), do)
+        assert np.array_equal(qt.cpu().numpy(), qo)
+        if qpad:                                           # nothing written between the rows
+            assert bool((qb[qoff:].view(rows, cols + qpad)[:, cols:] == 0xA5).all())
+    torch.cuda.synchronize()
+    assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("cols", [64, 1000, 4096, 4097, 8192, 16384, 16400])
+def test_grouped_rows_equal_single(gb, cols):
+    """fp8_quantize_e4m3_rows_grouped over matrices of mixed alignment and
+    length equals the single calls, for each register size it runs with."""
+    from paper_2602_10262_gb300._lib import FP8QuantJob
+    g = torch.Generator(device="cuda").manual_seed(cols)
+    mats, jobs, want = [], [], []
+    for rows, c, pad in ((3, cols, 0), (1, max(1, cols - 3), 1), (7, 17, 4)):
+        for aligned in (True, False):
+            x = torch.randn((rows, c + pad), generator=g, device="cuda")[:, :c]
+            q = torch.empty((rows, c + (0 if aligned else 1)), dtype=torch.uint8, device="cuda")[:, :c]
+            d = torch.empty(rows, device="cuda")
+            mats.append((x, q, d))
+            want.append(gb.fp8_quantize_e4m3(x, 1))
+            jobs.append(FP8QuantJob(x.data_ptr(), rows, c, x.stride(0), q.data_ptr(), q.stride(0), d.data_ptr()))
+    for subset in (slice(0, None), slice(0, 1)):
+        for _, q, d in mats:
+            q.zero_(), d.zero_()
+        arr = (FP8QuantJob * len(jobs[subset]))(*jobs[subset])
+        assert gb.library().fp8_quantize_e4m3_rows_grouped(arr, len(arr), torch.cuda.current_stream().cuda_stream) == 0
+        for (_, q, d), (qw, dw) in list(zip(mats, want))[subset]:
+            assert torch.equal(q, qw) and torch.equal(d, dw)
+    assert gb.fp8_last_device_error() == 0

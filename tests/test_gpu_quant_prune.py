@@ -95,3 +95,24 @@ def test_shape_and_alignment_rejected(gb):
     wide = torch.ones((4, 260), device="cuda")
     with pytest.raises(gb.Fp8Error):
         gb.fp8_quantize_e4m3_prune24(wide[:, 1:257])                # x not 16-byte aligned
+
+
+@pytest.mark.parametrize("rows", [5, 333])
+@pytest.mark.parametrize("cols", [128, 256, 384, 512, 640, 1024, 1152, 2048, 2176, 4096, 4224, 6144, 6272, 8192, 8320,
+                                  12288, 12416, 16384, 16512])
+def test_row_shapes(gb, rows, cols):
+    """Each threads-per-row shape at its first and last column counts, with
+    32- and 16-byte aligned x and 8- and 4-byte aligned outputs, equals the
+    two separate calls."""
+    g = torch.Generator(device="cuda").manual_seed(rows + cols)
+    for pad, off in ((0, 0), (4, 4)):
+        x = torch.randn(rows * (cols + pad) + off, generator=g, device="cuda")[off:].view(rows, cols + pad)[:, :cols]
+        q = torch.empty(rows * (cols + pad) + off, dtype=torch.uint8, device="cuda")[off:].view(
+            rows, cols + pad)[:, :cols]
+        v = torch.empty(rows * cols // 2 + off // 2, dtype=torch.uint8, device="cuda")[off // 2:].view(rows, cols // 2)
+        q, d, v, m = gb.fp8_quantize_e4m3_prune24(x, q=q, a_vals=v)
+        q2, d2 = gb.fp8_quantize_e4m3(x, 1)
+        v2, m2 = gb.prune24_compress(q2)
+        assert torch.equal(d, d2) and torch.equal(q, q2) and torch.equal(v, v2) and torch.equal(m, m2)
+    torch.cuda.synchronize()
+    assert gb.fp8_last_device_error() == 0
