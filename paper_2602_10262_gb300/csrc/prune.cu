@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kThreads) prune24_vec_kernel(const uint8_t* __
                                                                uint8_t* __restrict__ meta)
 {
     grid_launch_dependents();
+    grid_dependency_wait();
     const int pieces = static_cast<int>(K / 16);
     const int64_t ldv = K / 2, ldm = K / 8;
     const int p_first = blockIdx.x * (kThreads * U) + threadIdx.x;
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(kThreads) prune24_kernel(const uint8_t* __rest
                                                            uint8_t* __restrict__ meta)
 {
     grid_launch_dependents();
+    grid_dependency_wait();
     const int64_t ldv = K / 2, ldm = (K + 7) / 8;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     const int64_t tid = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x;
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(kThreads) decompress24_vec_kernel(const uint2*
                                                                     int64_t pieces, uint4* __restrict__ out)
 {
     grid_launch_dependents();
+    grid_dependency_wait();
     const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads * U);
     for (int64_t p0 = static_cast<int64_t>(blockIdx.x) * (kThreads * U) + threadIdx.x; p0 < pieces;
          p0 += step) {
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(kThreads) decompress24_kernel(const uint8_t* _
                                                                 uint8_t* __restrict__ out)
 {
     grid_launch_dependents();
+    grid_dependency_wait();
     const int64_t ldv = K / 2, ldm = (K + 7) / 8, groups = K / 4;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < M * groups;
@@ -209,11 +213,11 @@ extern "C" int prune24_compress(const uint8_t* a, int64_t M, int64_t K, int64_t 
         const unsigned gx = static_cast<unsigned>((pieces + kThreads * u - 1) / (kThreads * u));
         const unsigned gy = static_cast<unsigned>(M < 65535 ? M : 65535);
         if (u == 1)
-            prune24_vec_kernel<1><<<dim3(gx, gy), kThreads, 0, st>>>(a, M, K, lda, a_vals, a_meta);
+            launch_dependent(prune24_vec_kernel<1>, dim3(gx, gy), kThreads, st, a, M, K, lda, a_vals, a_meta);
         else
-            prune24_vec_kernel<kPieces><<<dim3(gx, gy), kThreads, 0, st>>>(a, M, K, lda, a_vals, a_meta);
+            launch_dependent(prune24_vec_kernel<kPieces>, dim3(gx, gy), kThreads, st, a, M, K, lda, a_vals, a_meta);
     } else {
-        prune24_kernel<<<grid_for(M * ((K + 7) / 8)), kThreads, 0, st>>>(a, M, K, lda, a_vals, a_meta);
+        launch_dependent(prune24_kernel, grid_for(M * ((K + 7) / 8)), kThreads, st, a, M, K, lda, a_vals, a_meta);
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
@@ -243,11 +247,11 @@ extern "C" int prune24_decompress(const uint8_t* a_vals, const uint8_t* a_meta, 
         const auto* m2 = reinterpret_cast<const uint16_t*>(a_meta);
         auto* o16 = reinterpret_cast<uint4*>(out);
         if (u == 1)
-            decompress24_vec_kernel<1><<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(v8, m2, pieces, o16);
+            launch_dependent(decompress24_vec_kernel<1>, static_cast<unsigned>(blocks), kThreads, st, v8, m2, pieces, o16);
         else
-            decompress24_vec_kernel<kPieces><<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(v8, m2, pieces, o16);
+            launch_dependent(decompress24_vec_kernel<kPieces>, static_cast<unsigned>(blocks), kThreads, st, v8, m2, pieces, o16);
     } else {
-        decompress24_kernel<<<grid_for(M * (K / 4)), kThreads, 0, st>>>(a_vals, a_meta, M, K, out);
+        launch_dependent(decompress24_kernel, grid_for(M * (K / 4)), kThreads, st, a_vals, a_meta, M, K, out);
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;

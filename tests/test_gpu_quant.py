@@ -150,3 +150,46 @@ def test_grouped_rows_equal_single(gb, cols):
         for (_, q, d), (qw, dw) in list(zip(mats, want))[subset]:
             assert torch.equal(q, qw) and torch.equal(d, dw)
     assert gb.fp8_last_device_error() == 0
+
+
+def test_dependent_launches_keep_stream_order(gb):
+    """Back-to-back calls whose buffers feed one another (the kernels are
+    launched with programmatic serialization): eager and from a captured
+    graph, every pass equals the calls made one by one."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn((64, 2048), generator=g, device="cuda")
+    w = torch.randn((512, 2048), generator=g, device="cuda")
+
+    def chain(x, sync=lambda: None):
+        outs, h = [], x
+        for _ in range(3):
+            A, dA = gb.fp8_quantize_e4m3(h, 1)
+            sync()
+            B, dB, v, m = gb.fp8_quantize_e4m3_prune24(w)
+            sync()
+            C = gb.gemm_fp8_dense(A, B, dA, 1, dB, 1, out_dtype=gb.OUT_F32)
+            sync()
+            P = gb.prune24_decompress(*gb.prune24_compress(B), 2048)
+            sync()
+            h = torch.cat([gb.gemm_fp8_dense(A, P, dA, 1, dB, 1, out_dtype=gb.OUT_F32), C, C, C], 1)
+            sync()
+            outs += [A, dA, C, h]
+        return outs
+
+    want = chain(x, torch.cuda.synchronize)
+    for _ in range(5):
+        assert all(torch.equal(a, b) for a, b in zip(chain(x), want))
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        chain(x)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = chain(x)
+    for _ in range(3):
+        for t in got:
+            t.zero_()
+        graph.replay()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert gb.fp8_last_device_error() == 0
