@@ -539,9 +539,11 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
         const int nck = cw * ESZ / 16;                   // 16-byte pieces per row
         const bool via_tma = tmC != nullptr && cw == CW;
         if (tmC != nullptr) {
-            // the store that last used this buffer (NB chunks ago) must have read it
+            // the store that last used this buffer (NB chunks ago; of any
+            // earlier call on a call's first chunk, whichever buffer it ended
+            // on) must have read it
             if (lane == 0) {
-                if (NB == 2)
+                if (NB == 2 && c0 != c_lo)
                     bulk_wait_read_1();
                 else
                     bulk_wait_read_all();
