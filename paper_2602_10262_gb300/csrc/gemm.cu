@@ -91,7 +91,18 @@ constexpr int SPARSE_BN_MAX_MT2 = 224;
 // chunk; a pair's CTA holds all 256 rows of B's), copied into a ring of
 // TMEM columns (per k-block A's 4, then 4 per 128 rows of B): columns
 // 128..255 beside the first of two accumulators for 128-wide tiles, from
-// column 256 after the single accumulator for 256-wide ones and pairs.
+// column 256 after the single accumulator for 256-wide ones and pairs
+// (MX = 1).  One accumulator stops the tensor pipe for every tile's
+// epilogue, so pairs with more than one tile each (MX = 2) keep a ring of
+// four k-blocks in the last 48 columns and two accumulators that share 48
+// columns in the 464 before it: columns 0..255 and 208..463.  Their epilogue
+// reads the 64 columns that hold the shared ones into registers first and
+// releases them, so the next tile's MMAs wait for that read only: 4096 x
+// 14336 x 4096 198 -> 173 us, 4096^3 67.7 -> 61.4 us, 8192^3 397 -> 385 us
+// (its k-loop is long; what is left there against 310 us for unscaled codes
+// is the scales' copies to tensor memory, 5 %, their loads, 4 %, and an
+// epilogue of four warps).  With one tile per pair nothing can overlap, and
+// the drain's code costs 1.8 of 20 us (1000 x 3000 x 4096): MX = 1.
 // PAIR: CTA-pair launches (cta_group::2, clusters of two): a 256 x 256 tile
 // per pair, each CTA loading its 128 rows of A and 128 rows of B (two
 // k-blocks per stage, three 64 KB stages) and holding its 128 x 256 half of
@@ -105,7 +116,7 @@ constexpr int SPARSE_BN_MAX_MT2 = 224;
 constexpr int PAIR_TMEM_COLS = 512;       // columns per CTA: two accumulators (the epilogue of
                                           // one tile overlaps the MMAs of the next)
 
-template <int MT, bool SP = false, int BNC = BN_MAX, int KC = 1, bool MX = false, bool PAIR = false>
+template <int MT, bool SP = false, int BNC = BN_MAX, int KC = 1, int MX = 0, bool PAIR = false>
 struct Cfg {
     static constexpr bool kSparse2 = MT == 2 && SP;
     static constexpr int kStages =
@@ -130,15 +141,20 @@ struct Cfg {
     // swizzle atoms
     static constexpr int kSfBytes = MX ? (KC * (1 + kSfQ) * kSfChunk + 1023) / 1024 * 1024 : 0;
     // MX: the scale ring's TMEM columns (per k-block 4 for A, 4 per 128 rows
-    // of B): beside the first accumulator for 128-wide tiles, after the
-    // single accumulator for 256-wide ones
+    // of B)
     static constexpr int kSfCols = 4 * (1 + kSfQ);
-    static constexpr int kSfCol0 = (MX && BNC == BN_MAX) ? BN_MAX : BNC;
+    // MX == 2: two accumulators with shared columns (see above)
+    static constexpr bool kOverlap = MX == 2;
+    static constexpr int kSfSlots = kOverlap ? 4 : kStages * KC;     // k-blocks of the scale ring
+    static constexpr int kSfCol0 = kOverlap ? TMEM_COLS - kSfCols * kSfSlots : BNC;     // (one 256-wide: after it)
+    // first column of accumulator 1, and columns drained before the release
+    static constexpr int kAcc1 = kOverlap ? kSfCol0 - BN_MAX : BN_MAX;
+    static constexpr int kDrainFirst = 64;
     static constexpr int kStageBytes = kABytes + kBBytes + kSfBytes;
     static constexpr int kMetaCol0 = kSparse2 ? SPARSE_BN_MAX_MT2 : (BNC == 256 ? SPARSE_BN_MAX : BNC);
     static constexpr int kTmemCols = PAIR ? PAIR_TMEM_COLS : TMEM_COLS;
     static constexpr int kAcc = (PAIR && !MX) ? PAIR_TMEM_COLS / BN_MAX
-                                              : ((MT == 2 || (MX && BNC == BN_MAX)) ? 1 : 2);   // accumulators
+                                              : ((MT == 2 || (MX == 1 && BNC == BN_MAX)) ? 1 : 2);   // accumulators
     // epilogue warps: 4 per 128 rows (one per TMEM lane quarter); 256-wide
     // 128-row tiles (and pairs) use 8, two per lane quarter splitting the
     // columns, so each SM sub-partition has a second warp to hide latencies
@@ -166,8 +182,12 @@ struct Cfg {
     static_assert(kBChunk % 1024 == 0, "B chunks stay swizzle-atom aligned");
     static_assert(!MX || (MT == 1 && !SP && (BNC == 128 || (BNC == BN_MAX && (KC == 1 || PAIR)))),
                   "block-scaled launches: 128-row dense tiles, 128 or 256 wide, or CTA pairs");
-    static_assert(!MX || kSfCol0 + kSfCols * kStages * KC <= (kAcc == 1 ? TMEM_COLS : BN_MAX),
+    static_assert(!MX || kSfCol0 + kSfCols * kSfSlots <= (kOverlap || kAcc == 1 ? TMEM_COLS : BN_MAX),
                   "scale ring fits beside the accumulators");
+    static_assert(!kOverlap || (kAcc1 >= BN_MAX - kDrainFirst && kAcc1 < BN_MAX),
+                  "the columns drained first hold every column the accumulators share");
+    static_assert(!kOverlap || (PAIR && KC == 2 && kSfSlots == 2 * KC && kStages >= 3),
+                  "shared accumulators: pairs, two stages' worth of scale slots (guarded in the MMA loop)");
 };
 
 // Everything of a problem but its tensor maps.  Each role thread copies this
@@ -204,8 +224,8 @@ struct Problem : ProblemScalars {
     CUtensorMap tmP;        // P [rows_p, K] codes, box {128, 128 * MT}
     CUtensorMap tmQ;        // Q [rows_q, K] codes, box {128, bn}
     CUtensorMap tmE;        // sparse: metadata [rows_p, K/8], box {16, 128 * MT}; block-scaled CTA
-                            // pairs: P's scale chunks [chunks][32][16 bytes], box {16, 32, KC}
-    CUtensorMap tmSFQ;      // block-scaled CTA pairs: Q's scale chunks, as tmE
+                            // pairs: P's scale chunks [row tiles][k-blocks][512 bytes], box of KC chunks
+    CUtensorMap tmSFQ;      // block-scaled CTA pairs: Q's scale chunks, box of KC chunks x the tile's row tiles
     CUtensorMap tmC;        // C [rows_p, rows_q] (row stride ldc), box {128 bytes, 32 rows}, 128-byte swizzle
 };
 
@@ -476,16 +496,19 @@ __device__ __forceinline__ void cluster_reduce_store(const ProblemScalars& P, co
 // buffer is written again.  A partial last chunk (bn not a multiple of the
 // chunk width) is copied out by the lanes, masked, so no store reaches the
 // next tile's columns.
-template <int ESZ, int LB, int NB>  // LB: 16-column TMEM loads in flight per wait (1 or 2); NB: staging buffers
+// LB: 16-column TMEM loads in flight per wait (1 or 2); NB: staging buffers;
+// HELD > 0: the HELD columns from c_lo are in `held` already (c_hi = c_lo +
+// HELD), nothing is read from tensor memory.
+template <int ESZ, int LB, int NB, int HELD = 0>
 __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P, uint32_t taddr, int row0,
                                                         float fi, int jbase, uint8_t* bufs, int lane,
                                                         ScaleWindows& sw, const CUtensorMap* tmC, int c_lo,
-                                                        int c_hi)
+                                                        int c_hi, const uint32_t (*held)[16] = nullptr)
 {
     constexpr int CW = 128 / ESZ;                     // columns per chunk
     const int rows_q = P.rows_q;
     int nb = 0;                                       // staging buffer of this chunk
-    for (int c0 = c_lo; c0 < c_hi; c0 += CW) {
+    const auto chunk = [&](const int c0, const int hq) {       // hq: the chunk's first held group of 16
         uint8_t* buf = bufs + nb * (32 * 128);
         nb = NB == 2 ? nb ^ 1 : 0;
         const int cw = min(CW, c_hi - c0);           // multiple of 16
@@ -511,7 +534,11 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
                 }
             }
         };
-        if constexpr (LB == 2) {
+        if constexpr (HELD > 0) {
+#pragma unroll
+            for (int q = 0; q < CW; q += 16)
+                convert16(held[hq + q / 16], q);
+        } else if constexpr (LB == 2) {
 #pragma unroll
             for (int q = 0; q < CW; q += 32) {
                 uint32_t ra[16], rb[16];
@@ -563,7 +590,7 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
                 tma_store_2d(tmC, smem_u32(buf), jbase + c0, row0);
                 bulk_commit();
             }
-            continue;
+            return;
         }
         __syncwarp();
         const int k = lane & 7;
@@ -586,12 +613,20 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
             }
         }
         __syncwarp();
+    };
+    if constexpr (HELD > 0) {
+#pragma unroll
+        for (int h = 0; h < HELD; h += CW)
+            chunk(c_lo + h, h / 16);
+    } else {
+        for (int c0 = c_lo; c0 < c_hi; c0 += CW)
+            chunk(c0, 0);
     }
 }
 
 // ---------------------------------------------------------------- kernel
 
-template <int MAXP, int MT, bool SP, int BNC, int KC, bool MX = false, bool PAIR = false>
+template <int MAXP, int MT, bool SP, int BNC, int KC, int MX = 0, bool PAIR = false>
 __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     gemm_fp8_kernel(const __grid_constant__ Params<MAXP> prm)
 {
@@ -816,12 +851,10 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                                                           (MX ? 2u * (1 + C::kSfQ) * KC * C::kSfChunk : 0u));
                         if constexpr (MX) {
                             const uint32_t sf = sa + C::kABytes + C::kBBytes;
-                            const int chunk_p = (tc.m_blk * 2 + static_cast<int>(rank)) * P.sf_kb + kb;
-                            tma_load_3d_pair(sf, &prm.prob[tc.p].tmE, fb, 0, 0, chunk_p);
-#pragma unroll
-                            for (int h = 0; h < C::kSfQ; ++h)
-                                tma_load_3d_pair(sf + (1 + h) * KC * C::kSfChunk, &prm.prob[tc.p].tmSFQ, fb, 0, 0,
-                                                 (tc.n_blk * C::kSfQ + h) * P.sf_kb + kb);
+                            tma_load_3d_pair(sf, &prm.prob[tc.p].tmE, fb, 0, kb,
+                                             tc.m_blk * 2 + static_cast<int>(rank));
+                            tma_load_3d_pair(sf + KC * C::kSfChunk, &prm.prob[tc.p].tmSFQ, fb, 0, kb,
+                                             tc.n_blk * C::kSfQ);
                         }
                         if constexpr (SP) {
                             // kept codes of the KC k-blocks, then their metadata
@@ -938,6 +971,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             int stage = 0;
             uint32_t phase = 0;
             int local = 0;
+            uint32_t sf_stage = 0;              // stages taken so far (scale ring of fewer slots)
             bool ok = true;
             // pairs: the even CTA issues the pair's MMAs
             const int mma_tiles = (PAIR && rank != 0) ? 0 : my_tiles;
@@ -949,18 +983,23 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 const uint32_t b_chunk = PAIR ? static_cast<uint32_t>(C::kBChunk)
                                               : static_cast<uint32_t>(P.bn) * BK;   // B chunks bn x 128 B apart
                 const int acc = local % C::kAcc;
-                const uint32_t acc_phase = (local / C::kAcc) & 1;
                 // an accumulator not used yet is free: no wait on its first use
-                // (pairs: both CTAs' epilogues release it, the odd one remotely)
-                if (local >= C::kAcc &&
-                    !(PAIR ? mbar_wait_cluster(tempty_bar(acc), acc_phase ^ 1u, abort_flag, wlim)
-                           : mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, wlim))) {
+                // (pairs: both CTAs' epilogues release it, the odd one
+                // remotely).  Accumulators with shared columns: one barrier,
+                // released once per tile when the shared columns are drained;
+                // tile n waits for tile n - 1's release, which its epilogue
+                // gives only after it has read all of tile n - 2.
+                const uint32_t tempty = tempty_bar(C::kOverlap ? 0 : acc);
+                const uint32_t freed = C::kOverlap ? (local - 1) & 1u : ((local / C::kAcc) & 1u) ^ 1u;
+                if (local >= (C::kOverlap ? 1 : C::kAcc) &&
+                    !(PAIR ? mbar_wait_cluster(tempty, freed, abort_flag, wlim)
+                           : mbar_wait(tempty, freed, abort_flag, wlim))) {
                     abort_pipeline(abort_flag, err);
                     break;
                 }
                 tc_fence_after();
                 // half h of the tile accumulates into columns d_tmem + 256 h
-                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * BN_MAX);
+                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * C::kAcc1);
                 const int kb0 = tc.slice * P.kb_per_split;
                 const int kb1 = min(P.k_blocks, kb0 + P.kb_per_split);
                 for (int kb = kb0; kb < kb1; kb += KC) {
@@ -972,7 +1011,22 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                         abort_pipeline(abort_flag, err);
                         break;
                     }
+                    if constexpr (C::kSfSlots < S * KC) {
+                        // the scale columns this stage is about to write were
+                        // last read by the MMAs of two stages ago: those are
+                        // done once their slot has been committed as empty (the
+                        // previous stage's MMAs, still running, hide this wait)
+                        if (sf_stage >= 2) {
+                            const int back = stage >= 2 ? stage - 2 : stage + S - 2;
+                            if (!mbar_wait(empty_bar(back), stage >= 2 ? phase : phase ^ 1u, abort_flag, wlim)) {
+                                ok = false;
+                                abort_pipeline(abort_flag, err);
+                                break;
+                            }
+                        }
+                    }
                     tc_fence_after();
+                    const int sf_slot = C::kSfSlots < S * KC ? (sf_stage++ & 1) * KC : stage * KC;
                     const uint32_t sa = smem_base + stage * C::kStageBytes;
                     if constexpr (PAIR) {
 #pragma unroll
@@ -1000,7 +1054,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                                 // tensor memory: A's 4 ring columns (the CTA's rows),
                                 // then B's 8 (all 256 rows of the tile)
                                 const uint32_t sf_col =
-                                    static_cast<uint32_t>(C::kSfCol0 + C::kSfCols * (stage * KC + c));
+                                    static_cast<uint32_t>(C::kSfCol0 + C::kSfCols * (sf_slot + c));
                                 const uint32_t sm_sf = sa + C::kABytes + C::kBBytes + c * C::kSfChunk;
                                 tmem_cp_32x128b_warpx4_pair(tmem_base + sf_col, sdesc_rows16_noswizzle(sm_sf));
 #pragma unroll
@@ -1037,7 +1091,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                             // time) -> their ring columns, each 32-row group to every
                             // lane quarter: B row r in column 4 + r / 32
                             const uint32_t sf_col =
-                                static_cast<uint32_t>(C::kSfCol0 + C::kSfCols * (stage * KC + c));
+                                static_cast<uint32_t>(C::kSfCol0 + C::kSfCols * (sf_slot + c));
                             const uint32_t sm_sf = sa + C::kABytes + C::kBBytes + c * C::kSfChunk;
                             tmem_cp_32x128b_warpx4(tmem_base + sf_col, sdesc_rows16_noswizzle(sm_sf));
 #pragma unroll
@@ -1158,6 +1212,15 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 c_lo = cpart ? mid : 0;
                 c_hi = cpart ? P.bn : mid;
             }
+            // accumulators with shared columns: those columns first (the top of
+            // accumulator 0, the bottom of accumulator 1), then the rest; not
+            // on the CTA's last tile, which no other waits for
+            const int c_end = c_hi;
+            const bool drain = C::kOverlap && tile + tile_step < my_tiles;
+            if (drain) {
+                c_lo = acc ? 0 : P.bn - C::kDrainFirst;
+                c_hi = c_lo + C::kDrainFirst;
+            }
             ScaleWindows sw;
             sw.init(P, jbase + c_lo, lane, c_hi - c_lo);
             // the whole warp takes the same branch (tcgen05.ld is warp-collective)
@@ -1168,7 +1231,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             }
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
-                                   static_cast<uint32_t>((acc + half) * BN_MAX);
+                                   static_cast<uint32_t>(acc * C::kAcc1 + half * BN_MAX);
             if (P.splits > 1 && cluster_split) {
                 const int crank = static_cast<int>(cluster_ctarank());
                 if (crank != tc.slice) {                // launch shape broken: never expected
@@ -1233,13 +1296,50 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 }
                 continue;
             }
+            const auto release = [&] {
+                tc_fence_before();
+                const uint32_t bar = tempty_bar(C::kOverlap ? 0 : acc);
+                if (PAIR && rank != 0)
+                    mbar_arrive_remote(cluster_map(bar, 0u));     // the even CTA's barrier
+                else
+                    mbar_arrive(bar);
+            };
+            uint8_t* buf = epi_smem + (warp - 2) * C::kEpiBufs * 32 * 128;
+            const int row0 = i - lane;
+            const CUtensorMap* tmC = P.tma_store ? &prm.prob[tc.p].tmC : nullptr;
+            // (kernels with 8 epilogue warps have the smaller register
+            // budget: one load per wait)
+            constexpr int LB = C::kEpiWarps == 4 ? 2 : 1;
+            if (drain) {
+                // the shared columns into registers, released before they are
+                // converted and stored
+                uint32_t held[C::kDrainFirst / 16][16];
+#pragma unroll
+                for (int h = 0; h < C::kDrainFirst / 16; ++h)
+                    tmem_ld_32x32b_x16(taddr + c_lo + 16 * h, held[h]);
+                tmem_ld_wait();
+                release();
+                if (!P.trans_out && P.vec_store) {
+                    if (P.out_bf16)
+                        epilogue_rows_coalesced<2, LB, C::kEpiBufs, C::kDrainFirst>(
+                            P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo, c_hi, held);
+                    else
+                        epilogue_rows_coalesced<4, LB, C::kEpiBufs, C::kDrainFirst>(
+                            P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo, c_hi, held);
+                } else {
+                    float s_cur = 0.0f;
+#pragma unroll
+                    for (int h = 0; h < C::kDrainFirst / 16; ++h) {
+                        if (h % 2 == 0)
+                            s_cur = sw.take(P, jbase + c_lo, lane);
+                        store_chunk16(P, i, row_ok, fi, jbase + c_lo + 16 * h, held[h], s_cur, 16 * (h & 1));
+                    }
+                }
+                c_lo = acc ? C::kDrainFirst : 0;
+                c_hi = acc ? c_end : c_end - C::kDrainFirst;
+                sw.init(P, jbase + c_lo, lane, c_hi - c_lo);
+            }
             if (!P.trans_out && P.vec_store) {
-                uint8_t* buf = epi_smem + (warp - 2) * C::kEpiBufs * 32 * 128;
-                const int row0 = i - lane;
-                const CUtensorMap* tmC = P.tma_store ? &prm.prob[tc.p].tmC : nullptr;
-                // (kernels with 8 epilogue warps have the smaller register
-                // budget: one load per wait)
-                constexpr int LB = C::kEpiWarps == 4 ? 2 : 1;
                 if (P.out_bf16)
                     epilogue_rows_coalesced<2, LB, C::kEpiBufs>(P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo,
                                                                c_hi);
@@ -1257,11 +1357,8 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                     store_chunk16(P, i, row_ok, fi, jbase + c0, r, s_cur, c0 & 31);
                 }
             }
-            tc_fence_before();
-            if (PAIR && rank != 0)
-                mbar_arrive_remote(cluster_map(tempty_bar(acc), 0u));     // the even CTA's barrier
-            else
-                mbar_arrive(tempty_bar(acc));
+            if (!drain)
+                release();
         }
         // TMA stores issued by this warp are complete before the CTA ends
         if (lane == 0)
@@ -1363,19 +1460,21 @@ bool make_map3(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, i
     return r == CUDA_SUCCESS;
 }
 
-// 3-D map over block-scale chunks viewed as [chunks][32][16 bytes] (the
-// tiled layout: 512 bytes per 128 rows x one k-block); box {16, 32, kc}
-// lands kc consecutive chunks as the contiguous bytes a bulk copy would.
-bool make_sf_map(CUtensorMap* map, const void* base, int64_t chunks, int kc)
+// 3-D map over tiled block scales as [128-row tiles][kb k-blocks][512 bytes]
+// (x in 32-bit words); box {512 bytes, kc, tiles}: one copy lands the kc
+// chunks of each of `tiles` row tiles back to back, as bulk copies would.
+// Whole 512-byte rows matter: [chunks][32][16 bytes] boxes, one per row tile
+// (five boxes a stage with the codes'), made 4096 x 14336 x 4096 2 % slower.
+bool make_sf_map(CUtensorMap* map, const void* base, int64_t row_tiles, int64_t kb, int kc, int tiles)
 {
     auto fn = encode_fn();
     if (!fn)
         return false;
-    cuuint64_t dims[3] = {16, 32, static_cast<cuuint64_t>(chunks)};
-    cuuint64_t strides[2] = {16, 512};
-    cuuint32_t box[3] = {16, 32, static_cast<cuuint32_t>(kc)};
+    cuuint64_t dims[3] = {128, static_cast<cuuint64_t>(kb), static_cast<cuuint64_t>(row_tiles)};
+    cuuint64_t strides[2] = {512, static_cast<cuuint64_t>(512 * kb)};
+    cuuint32_t box[3] = {128, static_cast<cuuint32_t>(kc), static_cast<cuuint32_t>(tiles)};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(base), dims, strides, box, estr,
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
@@ -1589,8 +1688,8 @@ int fill_problem(Problem& pr, const Job& j, int bn, int mt, int kc)
         pr.sf_kb = pr.k_blocks;
         // pairs load the scale chunks by TMA (their copies complete on the
         // even CTA's barrier); chunks past the arrays read as zeros
-        if (pair && (!make_sf_map(&pr.tmE, j.sfp, ((j.rows_p + BM - 1) / BM) * pr.sf_kb, kc) ||
-                     !make_sf_map(&pr.tmSFQ, j.sfq, ((j.rows_q + BM - 1) / BM) * pr.sf_kb, kc)))
+        if (pair && (!make_sf_map(&pr.tmE, j.sfp, (j.rows_p + BM - 1) / BM, pr.sf_kb, kc, 1) ||
+                     !make_sf_map(&pr.tmSFQ, j.sfq, (j.rows_q + BM - 1) / BM, pr.sf_kb, kc, bn / BM)))
             return FP8_ERR_CUDA;
     }
     return FP8_OK;
@@ -1648,7 +1747,7 @@ void bind_workspace(Params<MAXP>& prm, const Plan& pl, void* base)
     bind_workspace(prm, base, pl.ctr_count);
 }
 
-template <int MAXP, int MT, bool SP, int BNC = BN_MAX, int KC = 1, bool MX = false, bool PAIR = false>
+template <int MAXP, int MT, bool SP, int BNC = BN_MAX, int KC = 1, int MX = 0, bool PAIR = false>
 int plan(Params<MAXP>& prm, int max_ctas, Plan* out)
 {
     using C = Cfg<MT, SP, BNC, KC, MX, PAIR>;
@@ -1958,18 +2057,22 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
         // tiles (one accumulator, the scale ring after it) or 128 x 128
         // tiles (two)
         if constexpr (MAXP == 1) {
+            // pairs: two accumulators with shared columns once a pair takes a
+            // second tile (see the MX comment at Cfg)
             if (c.mt == 3)
-                return plan<MAXP, 1, false, BN_MAX, 2, true, true>(prm, max_ctas, pl);
+                return 2 * prm.prob[0].m_blocks * prm.prob[0].n_blocks > (max_ctas > 0 ? max_ctas : sm_count())
+                           ? plan<MAXP, 1, false, BN_MAX, 2, 2, true>(prm, max_ctas, pl)
+                           : plan<MAXP, 1, false, BN_MAX, 2, 1, true>(prm, max_ctas, pl);
             if (max_bn > 128)
-                return plan<MAXP, 1, false, BN_MAX, 1, true>(prm, max_ctas, pl);
-            return kc == 2 ? plan<MAXP, 1, false, 128, 2, true>(prm, max_ctas, pl)
-                           : plan<MAXP, 1, false, 128, 1, true>(prm, max_ctas, pl);
+                return plan<MAXP, 1, false, BN_MAX, 1, 1>(prm, max_ctas, pl);
+            return kc == 2 ? plan<MAXP, 1, false, 128, 2, 1>(prm, max_ctas, pl)
+                           : plan<MAXP, 1, false, 128, 1, 1>(prm, max_ctas, pl);
         }
         return FP8_ERR_UNSUPPORTED;
     }
     if (c.mt == 3)
-        return sparse ? plan<MAXP, 1, true, SPARSE_BN_MAX_MT2, 2, false, true>(prm, max_ctas, pl)
-                      : plan<MAXP, 1, false, BN_MAX, 2, false, true>(prm, max_ctas, pl);
+        return sparse ? plan<MAXP, 1, true, SPARSE_BN_MAX_MT2, 2, 0, true>(prm, max_ctas, pl)
+                      : plan<MAXP, 1, false, BN_MAX, 2, 0, true>(prm, max_ctas, pl);
     if (c.mt == 1) {
         if (kc == 2 && all_sparse) {
             if (max_bn <= 16)

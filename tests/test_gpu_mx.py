@@ -340,3 +340,34 @@ def test_mx_pairs_stalled_launch_times_out(gb):
     torch.cuda.synchronize()
     assert gb.fp8_last_device_error() == 0
     assert np.array_equal(C.cpu().numpy(), ref)
+
+
+# pairs with one tile each (one accumulator) and with several (accumulators
+# with shared columns): odd and even tile counts per pair, one k-block, an
+# odd number of k-blocks, a partial last k-block, an unaligned output
+@pytest.mark.parametrize("M,N,K,out", [(2560, 2560, 4096, 0), (5120, 2816, 128, 0), (5200, 2800, 416, 1),
+                                       (5120, 5001, 672, 0), (7680, 7680, 160, 1)])
+def test_mx_pair_tile_counts_exact(gb, M, N, K, out):
+    """Integers times powers of two: every partial sum is exact in FP32, so
+    the product equals float64's."""
+    A = _dev(workloads.small_int_codes((M, K), seed=M))
+    B = _dev(workloads.small_int_codes((N, K), seed=N + 1))
+    g = torch.Generator().manual_seed(K)
+
+    def scales(rows):
+        s = torch.randint(126, 129, (rows, K // 32), generator=g, dtype=torch.int32).to(torch.uint8).cuda()
+        return s, gb.fp8_mx_scales_to_tiled(s, rows, K)
+
+    def value(codes, s):
+        v = codes.view(torch.float8_e4m3fn).double().reshape(codes.shape[0], K // 32, 32)
+        return (v * torch.exp2(s.double() - 127)[:, :, None]).reshape(codes.shape)
+
+    (sa, ta), (sb, tb) = scales(M), scales(N)
+    assert gb.gemm_fp8_mx_plan(M, N, K, out)["mt"] == 3
+    C = gb.gemm_fp8_mx(A, ta, B, tb, out_dtype=out)
+    assert gb.fp8_last_device_error() == 0
+    ref = value(A, sa) @ value(B, sb).T
+    if out == gb.OUT_F32:
+        assert torch.equal(C.double(), ref)
+    else:
+        assert torch.equal(C, ref.float().bfloat16())
