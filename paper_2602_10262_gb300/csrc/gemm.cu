@@ -491,11 +491,12 @@ __device__ __forceinline__ void cluster_reduce_store(const ProblemScalars& P, co
 // The staging buffer of a warp is 32 rows x 128 bytes, 1024-aligned, with
 // 16-byte piece k of row r at (k ^ (r & 7)) * 16: the layout of a TMA box
 // {128 bytes, 32 rows} with 128-byte swizzle.  Full-width chunks leave
-// through one TMA store issued by lane 0 (which clips rows and columns
-// outside C); lane 0 waits until that store has read the buffer before the
+// through one TMA store issued by lane 0 (which clips rows outside C, and
+// columns to 16 bytes); lane 0 waits until that store has read the buffer before the
 // buffer is written again.  A partial last chunk (bn not a multiple of the
-// chunk width) is copied out by the lanes, masked, so no store reaches the
-// next tile's columns.
+// chunk width, or the end of rows that are not a multiple of 16 bytes) is
+// copied out by the lanes, masked, so no store reaches the next tile's
+// columns or past C's.
 // LB: 16-column TMEM loads in flight per wait (1 or 2); NB: staging buffers;
 // HELD > 0: the HELD columns from c_lo are in `held` already (c_hi = c_lo +
 // HELD), nothing is read from tensor memory.
@@ -509,6 +510,8 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
     const int rows_q = P.rows_q;
     int nb = 0;                                       // staging buffer of this chunk
     const auto chunk = [&](const int c0, const int hq) {       // hq: the chunk's first held group of 16
+        if (jbase + c0 >= rows_q)                     // no column of C (and the chunks after it)
+            return;
         uint8_t* buf = bufs + nb * (32 * 128);
         nb = NB == 2 ? nb ^ 1 : 0;
         const int cw = min(CW, c_hi - c0);           // multiple of 16
@@ -564,7 +567,11 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
             }
         }
         const int nck = cw * ESZ / 16;                   // 16-byte pieces per row
-        const bool via_tma = tmC != nullptr && cw == CW;
+        // a TMA store writes whole 16-byte pieces (the bytes past the last
+        // column of C's rows become zeros), so a chunk that holds the end of
+        // rows that are not a multiple of 16 bytes leaves through the lanes
+        const bool via_tma =
+            tmC != nullptr && cw == CW && ((rows_q * ESZ) % 16 == 0 || jbase + c0 + CW <= rows_q);
         if (tmC != nullptr) {
             // the store that last used this buffer (NB chunks ago; of any
             // earlier call on a call's first chunk, whichever buffer it ended

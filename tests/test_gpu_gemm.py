@@ -371,3 +371,25 @@ def test_grouped_long_list_equals_single_calls(gb, orc):
     assert gb.fp8_last_device_error() == 0
     for a, b in zip(outs, refs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("mt", [1, 2, 3])
+@pytest.mark.parametrize("N,ld", [(31, 32), (33, 64), (57, 64), (61, 64), (63, 64), (65, 72), (127, 128), (129, 256),
+                                  (250, 256), (255, 256), (257, 512)])
+def test_columns_past_the_output_untouched(gb, mt, out, N, ld):
+    """Aligned row strides with a column count that ends inside a 16-byte
+    piece: the columns between N and the stride keep their values."""
+    M, K = 300, 128
+    A = _cuda(workloads.small_int_codes((M, K), seed=1, maxabs=2))
+    B = _cuda(workloads.small_int_codes((N, K), seed=N, maxabs=2))
+    ref = (A.view(torch.float8_e4m3fn).double() @ B.view(torch.float8_e4m3fn).double().T).float()
+    gb.fp8_gemm_set_tile_config(mt, 0)
+    try:
+        C = torch.full((M, ld), 7.0, dtype=torch.bfloat16 if out else torch.float32, device="cuda")
+        gb.gemm_fp8_dense(A, B, _ones(), 0, _ones(), 0, 1.0, out, C=C[:, :N])
+    finally:
+        gb.fp8_gemm_set_tile_config(0, 0)
+    assert torch.equal(C[:, :N].float(), ref.to(C.dtype).float())
+    assert bool((C[:, N:] == 7).all())
+    assert gb.fp8_last_device_error() == 0
