@@ -393,3 +393,28 @@ def test_columns_past_the_output_untouched(gb, mt, out, N, ld):
     assert torch.equal(C[:, :N].float(), ref.to(C.dtype).float())
     assert bool((C[:, N:] == 7).all())
     assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("mt", [0, 2, 3])
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(130, 1, 128), (130, 17, 96), (160, 63, 128), (257, 65, 256), (300, 129, 128),
+                                   (520, 257, 128), (400, 513, 384), (4100, 1027, 256)])
+def test_rows_that_start_anywhere(gb, mt, out, M, N, K):
+    """Outputs whose rows start on any element (odd strides and offsets):
+    integers exact against float64, nothing written outside the matrix."""
+    A = _cuda(workloads.small_int_codes((M, K), seed=M, maxabs=2))
+    B = _cuda(workloads.small_int_codes((N, K), seed=N, maxabs=2))
+    ref = A.view(torch.float8_e4m3fn).double() @ B.view(torch.float8_e4m3fn).double().T
+    dt = torch.bfloat16 if out else torch.float32
+    ref = ref.float().to(dt)
+    gb.fp8_gemm_set_tile_config(mt, 0)
+    try:
+        for pad, off in ((0, 1), (1, 0), (2, 3), (3, 2)):
+            buf = torch.full((M * (N + pad) + off + 8,), 7.0, dtype=dt, device="cuda")
+            C = buf[off:off + M * (N + pad)].view(M, N + pad)
+            gb.gemm_fp8_dense(A, B, _ones(), 0, _ones(), 0, 1.0, out, C=C[:, :N])
+            assert torch.equal(C[:, :N], ref)
+            assert bool((C[:, N:] == 7).all()) and bool((buf[:off] == 7).all()) and bool((buf[-8:] == 7).all())
+    finally:
+        gb.fp8_gemm_set_tile_config(0, 0)
+    assert gb.fp8_last_device_error() == 0
