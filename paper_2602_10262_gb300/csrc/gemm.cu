@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     if (warp == 2 && lane == 0 && tile0 < total_tiles && !prm.withhold_loads) {
         const int bn = P_first.bn;
         const int prow0 = PAIR ? tc_first.m_blk * 2 * BM + BM * static_cast<int>(rank) : tc_first.m_blk * BM * MT;
-        const int pcol0 = tc_first.n_blk * bn + (PAIR ? (BNC / 2) * static_cast<int>(rank) : 0) +
+        const int pcol0 = tc_first.n_blk * bn + (PAIR ? (bn / 2) * static_cast<int>(rank) : 0) +
                           (mc > 0 ? qrank * (bn / (mc > 0 ? mc : 1)) : 0);
         const int kb0 = tc_first.slice * P_first.kb_per_split;
         const int kb1 = min(min(P_first.k_blocks, kb0 + P_first.kb_per_split), kb0 + PREFETCH_STAGES * KC);
@@ -870,7 +870,8 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 const CUtensorMap* map_e = &prm.prob[tc.p].tmE;
                 const bool sparse = P.sparse != 0;
                 const uint32_t a_bytes = sparse ? C::kSpChunk + C::kMetaChunk : C::kAChunk;
-                const uint32_t b_chunk = static_cast<uint32_t>(P.bn) * BK;      // B chunks bn x 128 B apart
+                // B chunks bn x 128 B apart (pairs: each CTA's half of that)
+                const uint32_t b_chunk = static_cast<uint32_t>(PAIR ? P.bn / 2 : P.bn) * BK;
                 const int row0 = tc.m_blk * BM * MT;
                 const int col0 = tc.n_blk * P.bn;
                 const int kb0 = tc.slice * P.kb_per_split;
@@ -890,12 +891,12 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                         // CTAs' copies complete on the even CTA's barrier
                         const uint32_t fb = rank == 0 ? full_bar(stage) : cluster_map(full_bar(stage), 0u);
                         const int prow0 = tc.m_blk * 2 * BM + BM * static_cast<int>(rank);
-                        const int pcol0 = tc.n_blk * P.bn + (BNC / 2) * static_cast<int>(rank);
+                        const int pcol0 = tc.n_blk * P.bn + (P.bn / 2) * static_cast<int>(rank);
                         // block-scaled: by TMA, completing on the same barrier, each
                         // CTA's scale chunks of its 128 rows of A and of both 128-row
                         // halves of the tile's B (KC k-blocks each)
                         if (rank == 0)
-                            mbar_arrive_expect_tx(fb, 2u * static_cast<uint32_t>(C::kAChunk + C::kBChunk) *
+                            mbar_arrive_expect_tx(fb, 2u * (static_cast<uint32_t>(C::kAChunk) + b_chunk) *
                                                               static_cast<uint32_t>(P.tma3d ? KC : nck) +
                                                           (MX ? 2u * (1 + C::kSfQ) * KC * C::kSfChunk : 0u));
                         if constexpr (MX) {
@@ -918,7 +919,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                             for (int c = 0; c < KC; ++c) {
                                 if (c < nck) {
                                     tma_load_2d_pair(sa + c * C::kAChunk, map_p, fb, (kb + c) * BK, prow0);
-                                    tma_load_2d_pair(sa + C::kABytes + c * C::kBChunk, map_q, fb, (kb + c) * BK,
+                                    tma_load_2d_pair(sa + C::kABytes + c * b_chunk, map_q, fb, (kb + c) * BK,
                                                      pcol0);
                                 }
                             }
@@ -1029,8 +1030,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 const ProblemScalars P = tile == tile0 ? P_first : prm.prob[tc.p];
                 const bool sparse = P.sparse != 0;
                 const uint32_t idesc = P.idesc;
-                const uint32_t b_chunk = PAIR ? static_cast<uint32_t>(C::kBChunk)
-                                              : static_cast<uint32_t>(P.bn) * BK;   // B chunks bn x 128 B apart
+                const uint32_t b_chunk = static_cast<uint32_t>(PAIR ? P.bn / 2 : P.bn) * BK;
                 const int acc = local % C::kAcc;
                 // an accumulator not used yet is free: no wait on its first use
                 // (pairs: both CTAs' epilogues release it, the odd one
@@ -2069,6 +2069,43 @@ TileChoice choose(const Job* jobs, const int* bns, int n, int max_ctas, const Ti
     return c;
 }
 
+// N width of the CTA-pair tiles of a one-problem launch, up to `widest` (256
+// dense, 224 2:4).  Tiles run in waves of `pairs`, and a last wave that is
+// nearly empty costs as much as a full one, so the width with the least
+// waves x time per tile is taken; it has to save 5 % of the launch, since a
+// narrower tile reads A more often.  Time per tile and 128-wide k-block, in
+// cycles, fitted to a sweep of widths 112..256 over nine products (512 to
+// 4096 rows, K 4096 to 14336): it falls with the width far less than the
+// MMAs do, the loads of A and their latency being the rest.  Results do not
+// depend on the width: a column's sum is its own.  Measured against full
+// width, L2-cold: 512 x 12288 x 4096 27.0 -> 24.9 us (176 wide: two full
+// waves instead of one and a quarter), 2048 x 5120 x 4096 35.5 -> 34.1, 2:4
+// 512 x 14336 x 4096 33.1 -> 28.3; a wave more than needed loses as much
+// (4096^3: 45.5 us at 224, 51.1 at 208), and a narrower tile in the same one
+// wave gains nothing (512 x 8192 x 8192 at 224).
+int pair_width(const Job& j, int widest, int pairs)
+{
+    const bool sparse = j.E != nullptr;
+    const int64_t m_blocks = (j.rows_p + 2 * BM - 1) / (2 * BM);
+    const double k_blocks = static_cast<double>((j.K + BK - 1) / BK);
+    constexpr double kLaunch = 12400;             // cycles of a launch beside its tiles (6 us)
+    const auto cost = [&](int w) {
+        const int64_t tiles = m_blocks * ((j.rows_q + w - 1) / w);
+        const int64_t waves = (tiles + pairs - 1) / pairs;
+        const double block = sparse ? 318 + 1.26 * w : 462 + 0.78 * w;
+        return kLaunch + static_cast<double>(waves) * k_blocks * block;
+    };
+    int best = widest;
+    double best_cost = 0.95 * cost(widest);
+    for (int w = widest - 16; w >= 128; w -= 16) {
+        if (cost(w) < best_cost) {
+            best = w;
+            best_cost = cost(w);
+        }
+    }
+    return best;
+}
+
 // Fill the table for `n` jobs and plan the kernel variant that fits them.
 template <int MAXP>
 int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int max_ctas,
@@ -2095,6 +2132,9 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
         int bn = bns[i];
         if ((c.mt == 2 || c.mt == 3) && sparse)
             bn = std::min(bn, SPARSE_BN_MAX_MT2);
+        // (a tile kind forced process-wide keeps its full width)
+        if (c.mt == 3 && n == 1 && jobs[0].sfp == nullptr && g_force_mt.load(std::memory_order_relaxed) == 0)
+            bn = pair_width(jobs[0], bn, std::max(1, (max_ctas > 0 ? max_ctas : sm_count()) / 2));
         int rc = fill_problem(prm.prob[i], jobs[i], bn, c.mt, kc);
         if (rc != FP8_OK)
             return rc;

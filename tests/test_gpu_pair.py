@@ -210,3 +210,40 @@ def test_single_cta_cap_takes_no_pairs(gb, orc):
         assert gb.fp8_last_device_error() == 0
         outs.append(C)
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+@pytest.mark.parametrize("sparse", [False, True])
+@pytest.mark.parametrize("M,N,K", [(512, 12288, 4096), (1000, 3001, 4096), (2048, 5120, 4096), (4096, 4096, 1024),
+                                   (520, 11000, 4224), (14336, 512, 4096), (9000, 700, 4096)])
+def test_narrow_pair_tiles_equal_full_width(gb, sparse, M, N, K):
+    """The width a one-problem pair launch chooses for its waves changes no
+    bit, and the whole output is written (ragged rows, columns and k-blocks)."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    A, dA, v, m = gb.fp8_quantize_e4m3_prune24(torch.randn((M, K), generator=g, device="cuda"))
+    B, dB = gb.fp8_quantize_e4m3(torch.randn((N, K), generator=g, device="cuda"), 1)
+
+    def run(out):
+        C = torch.full((M, N), float("nan"), dtype=torch.bfloat16 if out else torch.float32, device="cuda")
+        if sparse:
+            return gb.gemm_fp8_sparse24(v, m, B, dA, 1, dB, 1, out_dtype=out, C=C)
+        return gb.gemm_fp8_dense(A, B, dA, 1, dB, 1, out_dtype=out, C=C)
+
+    for out in (0, 1):
+        got = run(out)
+        gb.fp8_gemm_set_tile_config(3, 0)
+        try:
+            full = run(out)
+        finally:
+            gb.fp8_gemm_set_tile_config(0, 0)
+        assert torch.equal(got, full)
+    assert gb.fp8_last_device_error() == 0
+
+
+def test_narrow_pair_tiles_are_planned(gb):
+    """Widths below the full one where it saves a wave's worth of time, full
+    width where it does not."""
+    narrow = [gb.gemm_fp8_dense_plan(M, N, K) for M, N, K in ((512, 12288, 4096), (2048, 5120, 4096))]
+    assert all(p["mt"] == 3 and 128 <= p["bn"] < 256 and p["bn"] % 16 == 0 for p in narrow), narrow
+    assert gb.gemm_fp8_dense_plan(16384, 16384, 16384)["bn"] == 256
+    assert gb.gemm_fp8_sparse24_plan(14336, 512, 4096)["bn"] < 224
+    assert gb.gemm_fp8_sparse24_plan(16384, 16384, 16384)["bn"] == 224
