@@ -56,6 +56,25 @@ def _stream(stream) -> ctypes.c_void_p:
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+# The calls below check and marshal every argument on each call; on a small
+# problem that is the call's whole time, so they read each attribute once and
+# pass plain integers.  Measured on the GB300 host (a 16 x 256 x 512 GEMM with
+# its output allocated): 11.7 us a call, 20.0 before; building a Stream object
+# for the current stream alone took 2.8.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream_ptr(stream) -> int:
+    """The stream's handle; None: the current stream of the current device
+    (CUDA is initialised: the caller holds a CUDA tensor)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and _raw_device is not None:
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
 def _dev(t: torch.Tensor, name: str, dtype: torch.dtype, dims: int):
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
@@ -65,6 +84,18 @@ def _dev(t: torch.Tensor, name: str, dtype: torch.dtype, dims: int):
         raise ValueError(f"{name} must have {dims} dimensions")
     if dims == 2 and t.numel() > 0 and t.stride(1) != 1:
         raise ValueError(f"{name} must have a contiguous last dimension")
+
+
+def _matrix(t, name: str, dtype: torch.dtype):
+    """(rows, columns, row stride, address) of a 2-D CUDA matrix of dtype."""
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.dim() == 2:
+        ld, step = t.stride()
+        if step == 1:
+            rows, cols = t.shape
+            return rows, cols, ld, t.data_ptr()
+    _dev(t, name, dtype, 2)                    # raises, or an empty matrix of any strides
+    rows, cols = t.shape
+    return rows, cols, t.stride(0), t.data_ptr()
 
 
 def _shape(t: torch.Tensor, name: str, shape) -> None:
@@ -80,12 +111,24 @@ def _packed(t: torch.Tensor, name: str) -> None:
         raise ValueError(f"{name} must be contiguous")
 
 
-def _scale(t, name: str, n: int) -> None:
-    """A scale vector: float32 on the GPU, contiguous, at least n entries."""
+def _packed_bytes(t, name: str, rows: int, cols: int) -> int:
+    """A contiguous uint8 CUDA matrix of exactly [rows, cols].  Its address."""
+    r, c, _, p = _matrix(t, name, torch.uint8)
+    if r != rows or c != cols:
+        _shape(t, name, (rows, cols))
+    _packed(t, name)
+    return p
+
+
+def _scale(t, name: str, n: int) -> int:
+    """A scale vector: float32 on the GPU, contiguous, at least n entries.  Its address."""
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is torch.float32 and t.numel() >= n and t.is_contiguous():
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != torch.float32:
         raise TypeError(f"{name} must be a float32 CUDA tensor")
     if not t.is_contiguous() or t.numel() < n:
         raise ValueError(f"{name} must be contiguous with at least {n} entries, got {t.numel()}")
+    return t.data_ptr()
 
 
 def _ld(t: torch.Tensor) -> int:
@@ -155,18 +198,19 @@ def fp8_gemm_set_multicast(mode: int = 0) -> None:
 
 
 def _quantize(name: str, x, scale_mode, q, dequant_scale, stream):
-    _dev(x, "x", torch.float32, 2)
-    R, C = x.shape
+    R, C, ldx, xp = _matrix(x, "x", torch.float32)
+    n = 1 if scale_mode == 0 else R
     if q is None:
         q = torch.empty((R, C), dtype=torch.uint8, device=x.device)
     if dequant_scale is None:
-        dequant_scale = torch.empty((1 if scale_mode == 0 else R,), dtype=torch.float32, device=x.device)
-    _dev(q, "q", torch.uint8, 2)
-    _shape(q, "q", (R, C))
-    _scale(dequant_scale, "dequant_scale", 1 if scale_mode == 0 else R)
-    rc = getattr(library(), name)(_p(x), R, C, _ld(x), int(scale_mode), _p(q), _ld(q),
-                                  _p(dequant_scale), _stream(stream))
-    _check(rc, name)
+        dequant_scale = torch.empty((n,), dtype=torch.float32, device=x.device)
+    qr, qc, ldq, qp = _matrix(q, "q", torch.uint8)
+    if qr != R or qc != C:
+        _shape(q, "q", (R, C))
+    dp = _scale(dequant_scale, "dequant_scale", n)
+    rc = getattr(_lib.load(), name)(xp, R, C, ldx, int(scale_mode), qp, ldq, dp, _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, name)
     return q, dequant_scale
 
 
@@ -190,8 +234,7 @@ def fp8_quantize_e4m3_prune24(x: torch.Tensor, q: Optional[torch.Tensor] = None,
     scales [R], kept codes [R, C/2], metadata [R, C/8]): per-row
     quantisation and the 2:4 compression of its codes in one pass, bitwise
     fp8_quantize_e4m3(x, 1) followed by prune24_compress."""
-    _dev(x, "x", torch.float32, 2)
-    R, C = x.shape
+    R, C, ldx, xp = _matrix(x, "x", torch.float32)
     dev = x.device
     if q is None:
         q = torch.empty((R, C), dtype=torch.uint8, device=dev)
@@ -201,16 +244,15 @@ def fp8_quantize_e4m3_prune24(x: torch.Tensor, q: Optional[torch.Tensor] = None,
         a_vals = torch.empty((R, C // 2), dtype=torch.uint8, device=dev)
     if a_meta is None:
         a_meta = torch.empty((R, C // 8), dtype=torch.uint8, device=dev)
-    _dev(q, "q", torch.uint8, 2)
-    _shape(q, "q", (R, C))
-    _scale(dequant_scale, "dequant_scale", R)
-    for t, nm, shp in ((a_vals, "a_vals", (R, C // 2)), (a_meta, "a_meta", (R, C // 8))):
-        _dev(t, nm, torch.uint8, 2)
-        _shape(t, nm, shp)
-        _packed(t, nm)
-    rc = library().fp8_quantize_e4m3_prune24(_p(x), R, C, _ld(x), _p(q), _ld(q), _p(dequant_scale),
-                                             _p(a_vals), _p(a_meta), _stream(stream))
-    _check(rc, "fp8_quantize_e4m3_prune24")
+    qr, qc, ldq, qp = _matrix(q, "q", torch.uint8)
+    if qr != R or qc != C:
+        _shape(q, "q", (R, C))
+    dp = _scale(dequant_scale, "dequant_scale", R)
+    rc = _lib.load().fp8_quantize_e4m3_prune24(xp, R, C, ldx, qp, ldq, dp,
+                                               _packed_bytes(a_vals, "a_vals", R, C // 2),
+                                               _packed_bytes(a_meta, "a_meta", R, C // 8), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "fp8_quantize_e4m3_prune24")
     return q, dequant_scale, a_vals, a_meta
 
 
@@ -225,23 +267,25 @@ def fp8_quantize_mx(x: torch.Tensor, fmt: int = E4M3, scale_layout: int = 1,
     """Block-scaled quantisation: fp32 [R, C] (C % 32 == 0) -> (codes uint8
     [R, C], E8M0 scale codes: uint8 [R, C / 32] for scale_layout 0, the tiled
     bytes gemm_fp8_mx reads for scale_layout 1)."""
-    _dev(x, "x", torch.float32, 2)
-    R, C = x.shape
+    R, C, ldx, xp = _matrix(x, "x", torch.float32)
     if q is None:
         q = torch.empty((R, C), dtype=torch.uint8, device=x.device)
-    _dev(q, "q", torch.uint8, 2)
-    _shape(q, "q", (R, C))
+    qr, qc, ldq, qp = _matrix(q, "q", torch.uint8)
+    if qr != R or qc != C:
+        _shape(q, "q", (R, C))
+    lib = _lib.load()
     if scale_layout == 0:
         shape = (R, C // 32)
     else:
-        shape = (fp8_mx_scale_tiled_bytes(R, C),)
+        shape = (lib.fp8_mx_scale_tiled_bytes(R, C),)
     if scales is None:
         scales = torch.empty(shape, dtype=torch.uint8, device=x.device)
     _shape(scales, "scales", shape)
     _packed(scales, "scales")
-    rc = library().fp8_quantize_mx(_p(x), R, C, _ld(x), int(fmt), _p(q), _ld(q), _p(scales),
-                                   int(scale_layout), _stream(stream))
-    _check(rc, "fp8_quantize_mx")
+    rc = lib.fp8_quantize_mx(xp, R, C, ldx, int(fmt), qp, ldq, scales.data_ptr(), int(scale_layout),
+                             _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "fp8_quantize_mx")
     return q, scales
 
 
@@ -265,41 +309,38 @@ def gemm_fp8_mx(A: torch.Tensor, a_scales: torch.Tensor, B: torch.Tensor, b_scal
                 b_format: int = E4M3, C: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Block-scaled GEMM: C[M, N] = alpha * sum_b 2^sa 2^sb dec(A) dec(B)^T over
     32-element blocks; a_scales / b_scales in the tiled layout."""
-    _dev(A, "A", torch.uint8, 2)
-    _dev(B, "B", torch.uint8, 2)
-    M, K = A.shape
-    N = B.shape[0]
-    if B.shape[1] != K:
+    M, K, lda, ap = _matrix(A, "A", torch.uint8)
+    N, Kb, ldb, bp = _matrix(B, "B", torch.uint8)
+    if Kb != K:
         raise ValueError("K mismatch")
+    lib = _lib.load()
     for t, nm, rows in ((a_scales, "a_scales", M), (b_scales, "b_scales", N)):
-        if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != torch.uint8:
+        if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype is not torch.uint8:
             raise TypeError(f"{nm} must be a uint8 CUDA tensor")
         _packed(t, nm)
-        if t.numel() < fp8_mx_scale_tiled_bytes(rows, K):
-            raise ValueError(f"{nm} must hold {fp8_mx_scale_tiled_bytes(rows, K)} bytes")
-    C = _out(C, M, N, out_dtype, A.device)
-    rc = library().gemm_fp8_mx(M, N, K, _p(A), _ld(A), _p(a_scales), _p(B), _ld(B), _p(b_scales),
-                               float(alpha), _p(C), _ld(C), int(out_dtype), int(a_format), int(b_format),
-                               _stream(stream))
-    _check(rc, "gemm_fp8_mx")
+        need = lib.fp8_mx_scale_tiled_bytes(rows, K)
+        if t.numel() < need:
+            raise ValueError(f"{nm} must hold {need} bytes")
+    C, ldc, cp = _out(C, M, N, out_dtype, A.device)
+    rc = lib.gemm_fp8_mx(M, N, K, ap, lda, a_scales.data_ptr(), bp, ldb, b_scales.data_ptr(), float(alpha), cp, ldc,
+                         int(out_dtype), int(a_format), int(b_format), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "gemm_fp8_mx")
     return C
 
 
 def prune24_compress(a: torch.Tensor, a_vals: Optional[torch.Tensor] = None,
                      a_meta: Optional[torch.Tensor] = None, stream=None):
     """E4M3 codes [M, K] -> (kept codes [M, K/2], metadata [M, ceil(K/8)])."""
-    _dev(a, "a", torch.uint8, 2)
-    M, K = a.shape
+    M, K, lda, ap = _matrix(a, "a", torch.uint8)
     if a_vals is None:
         a_vals = torch.empty((M, K // 2), dtype=torch.uint8, device=a.device)
     if a_meta is None:
         a_meta = torch.empty((M, (K + 7) // 8), dtype=torch.uint8, device=a.device)
-    for t, nm, shp in ((a_vals, "a_vals", (M, K // 2)), (a_meta, "a_meta", (M, (K + 7) // 8))):
-        _dev(t, nm, torch.uint8, 2)
-        _shape(t, nm, shp)
-        _packed(t, nm)
-    rc = library().prune24_compress(_p(a), M, K, _ld(a), _p(a_vals), _p(a_meta), _stream(stream))
-    _check(rc, "prune24_compress")
+    rc = _lib.load().prune24_compress(ap, M, K, lda, _packed_bytes(a_vals, "a_vals", M, K // 2),
+                                      _packed_bytes(a_meta, "a_meta", M, (K + 7) // 8), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "prune24_compress")
     return a_vals, a_meta
 
 
@@ -310,28 +351,27 @@ def prune24_decompress(a_vals: torch.Tensor, a_meta: torch.Tensor, K: int,
     M = a_vals.shape[0]
     if out is None:
         out = torch.empty((M, K), dtype=torch.uint8, device=a_vals.device)
-    for t, nm, shp in ((a_vals, "a_vals", (M, K // 2)), (a_meta, "a_meta", (M, (K + 7) // 8)),
-                       (out, "out", (M, K))):
-        _dev(t, nm, torch.uint8, 2)
-        _shape(t, nm, shp)
-        _packed(t, nm)
-    rc = library().prune24_decompress(_p(a_vals), _p(a_meta), M, K, _p(out), _stream(stream))
-    _check(rc, "prune24_decompress")
+    rc = _lib.load().prune24_decompress(_packed_bytes(a_vals, "a_vals", M, K // 2),
+                                        _packed_bytes(a_meta, "a_meta", M, (K + 7) // 8), M, K,
+                                        _packed_bytes(out, "out", M, K), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "prune24_decompress")
     return out
 
 
 def _out(C, rows, cols, out_dtype, device):
+    """The output (allocated when None is given), its row stride and address."""
     dt = torch.bfloat16 if out_dtype == OUT_BF16 else torch.float32
     if C is None:
         C = torch.empty((rows, cols), dtype=dt, device=device)
-    _dev(C, "C", dt, 2)
-    _shape(C, "C", (rows, cols))
-    return C
+    r, c, ldc, p = _matrix(C, "C", dt)
+    if r != rows or c != cols:
+        _shape(C, "C", (rows, cols))
+    return C, ldc, p
 
 
-def _scales(a_scale, a_mode, M, b_scale, b_mode, N) -> None:
-    _scale(a_scale, "a_scale", M if a_mode else 1)
-    _scale(b_scale, "b_scale", N if b_mode else 1)
+def _scales(a_scale, a_mode, M, b_scale, b_mode, N):
+    return _scale(a_scale, "a_scale", M if a_mode else 1), _scale(b_scale, "b_scale", N if b_mode else 1)
 
 
 def _sparse_a(a_vals, a_meta, M, K) -> None:
@@ -345,19 +385,7 @@ def gemm_fp8_dense(A: torch.Tensor, B: torch.Tensor, a_scale: torch.Tensor, a_mo
                    out_dtype: int = OUT_BF16, C: Optional[torch.Tensor] = None,
                    stream=None) -> torch.Tensor:
     """C[M, N] = alpha * sa * sb * dec(A)[M, K] @ dec(B)[N, K]^T."""
-    _dev(A, "A", torch.uint8, 2)
-    _dev(B, "B", torch.uint8, 2)
-    M, K = A.shape
-    N = B.shape[0]
-    if B.shape[1] != K:
-        raise ValueError("K mismatch")
-    C = _out(C, M, N, out_dtype, A.device)
-    _scales(a_scale, a_mode, M, b_scale, b_mode, N)
-    rc = library().gemm_fp8_dense(M, N, K, _p(A), _ld(A), _p(B), _ld(B), _p(a_scale), int(a_mode),
-                                  _p(b_scale), int(b_mode), float(alpha), _p(C), _ld(C),
-                                  int(out_dtype), _stream(stream))
-    _check(rc, "gemm_fp8_dense")
-    return C
+    return _dense("gemm_fp8_dense", A, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype, E4M3, E4M3, C, stream)
 
 
 def gemm_fp8_dense_fmt(A: torch.Tensor, B: torch.Tensor, a_scale: torch.Tensor, a_mode: int,
@@ -365,19 +393,21 @@ def gemm_fp8_dense_fmt(A: torch.Tensor, B: torch.Tensor, a_scale: torch.Tensor, 
                        out_dtype: int = OUT_BF16, a_format: int = E4M3, b_format: int = E4M3,
                        C: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """gemm_fp8_dense with A's codes read as a_format and B's as b_format."""
-    _dev(A, "A", torch.uint8, 2)
-    _dev(B, "B", torch.uint8, 2)
-    M, K = A.shape
-    N = B.shape[0]
-    if B.shape[1] != K:
+    return _dense("gemm_fp8_dense_fmt", A, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype, a_format, b_format,
+                  C, stream)
+
+
+def _dense(where, A, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype, a_format, b_format, C, stream):
+    M, K, lda, ap = _matrix(A, "A", torch.uint8)
+    N, Kb, ldb, bp = _matrix(B, "B", torch.uint8)
+    if Kb != K:
         raise ValueError("K mismatch")
-    C = _out(C, M, N, out_dtype, A.device)
-    _scales(a_scale, a_mode, M, b_scale, b_mode, N)
-    rc = library().gemm_fp8_dense_fmt(M, N, K, _p(A), _ld(A), _p(B), _ld(B), _p(a_scale),
-                                      int(a_mode), _p(b_scale), int(b_mode), float(alpha), _p(C),
-                                      _ld(C), int(out_dtype), int(a_format), int(b_format),
-                                      _stream(stream))
-    _check(rc, "gemm_fp8_dense_fmt")
+    C, ldc, cp = _out(C, M, N, out_dtype, A.device)
+    sa, sb = _scales(a_scale, a_mode, M, b_scale, b_mode, N)
+    rc = _lib.load().gemm_fp8_dense_fmt(M, N, K, ap, lda, bp, ldb, sa, int(a_mode), sb, int(b_mode), float(alpha), cp,
+                                        ldc, int(out_dtype), int(a_format), int(b_format), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, where)
     return C
 
 
@@ -386,23 +416,8 @@ def gemm_fp8_sparse24(a_vals: torch.Tensor, a_meta: torch.Tensor, B: torch.Tenso
                       alpha: float = 1.0, out_dtype: int = OUT_BF16, out_transposed: bool = False,
                       C: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Same product with A given as (a_vals [M, K/2], a_meta [M, K/8])."""
-    _dev(a_vals, "a_vals", torch.uint8, 2)
-    _dev(a_meta, "a_meta", torch.uint8, 2)
-    _dev(B, "B", torch.uint8, 2)
-    M = a_vals.shape[0]
-    K = a_vals.shape[1] * 2
-    N = B.shape[0]
-    if B.shape[1] != K:
-        raise ValueError("K mismatch")
-    C = _out(C, N if out_transposed else M, M if out_transposed else N, out_dtype, B.device)
-    _scales(a_scale, a_mode, M, b_scale, b_mode, N)
-    _sparse_a(a_vals, a_meta, M, K)
-    rc = library().gemm_fp8_sparse24(M, N, K, _p(a_vals), _p(a_meta), _p(B), _ld(B), _p(a_scale),
-                                     int(a_mode), _p(b_scale), int(b_mode), float(alpha), _p(C),
-                                     _ld(C), int(out_dtype), int(bool(out_transposed)),
-                                     _stream(stream))
-    _check(rc, "gemm_fp8_sparse24")
-    return C
+    return _sparse24("gemm_fp8_sparse24", a_vals, a_meta, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype,
+                     out_transposed, E4M3, E4M3, C, stream)
 
 
 def gemm_fp8_sparse24_fmt(a_vals: torch.Tensor, a_meta: torch.Tensor, B: torch.Tensor,
@@ -412,23 +427,26 @@ def gemm_fp8_sparse24_fmt(a_vals: torch.Tensor, a_meta: torch.Tensor, B: torch.T
                           b_format: int = E4M3, C: Optional[torch.Tensor] = None,
                           stream=None) -> torch.Tensor:
     """gemm_fp8_sparse24 with the kept codes of A read as a_format and B as b_format."""
-    _dev(a_vals, "a_vals", torch.uint8, 2)
-    _dev(a_meta, "a_meta", torch.uint8, 2)
-    _dev(B, "B", torch.uint8, 2)
-    M = a_vals.shape[0]
-    K = a_vals.shape[1] * 2
-    N = B.shape[0]
-    if B.shape[1] != K:
+    return _sparse24("gemm_fp8_sparse24_fmt", a_vals, a_meta, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype,
+                     out_transposed, a_format, b_format, C, stream)
+
+
+def _sparse24(where, a_vals, a_meta, B, a_scale, a_mode, b_scale, b_mode, alpha, out_dtype, out_transposed, a_format,
+              b_format, C, stream):
+    M, kept, _, vp = _matrix(a_vals, "a_vals", torch.uint8)
+    _, _, _, mp = _matrix(a_meta, "a_meta", torch.uint8)
+    N, Kb, ldb, bp = _matrix(B, "B", torch.uint8)
+    K = kept * 2
+    if Kb != K:
         raise ValueError("K mismatch")
-    C = _out(C, N if out_transposed else M, M if out_transposed else N, out_dtype, B.device)
-    _scales(a_scale, a_mode, M, b_scale, b_mode, N)
+    C, ldc, cp = _out(C, N if out_transposed else M, M if out_transposed else N, out_dtype, B.device)
+    sa, sb = _scales(a_scale, a_mode, M, b_scale, b_mode, N)
     _sparse_a(a_vals, a_meta, M, K)
-    rc = library().gemm_fp8_sparse24_fmt(M, N, K, _p(a_vals), _p(a_meta), _p(B), _ld(B),
-                                         _p(a_scale), int(a_mode), _p(b_scale), int(b_mode),
-                                         float(alpha), _p(C), _ld(C), int(out_dtype),
-                                         int(bool(out_transposed)), int(a_format), int(b_format),
-                                         _stream(stream))
-    _check(rc, "gemm_fp8_sparse24_fmt")
+    rc = _lib.load().gemm_fp8_sparse24_fmt(M, N, K, vp, mp, bp, ldb, sa, int(a_mode), sb, int(b_mode), float(alpha),
+                                           cp, ldc, int(out_dtype), int(bool(out_transposed)), int(a_format),
+                                           int(b_format), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, where)
     return C
 
 

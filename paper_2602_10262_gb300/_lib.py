@@ -146,6 +146,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Load (building first if needed) and return the CDLL."""
     global _lib
+    if _lib is not None:                       # set once, fully prepared, under the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
