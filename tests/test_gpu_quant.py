@@ -193,3 +193,42 @@ def test_dependent_launches_keep_stream_order(gb):
         graph.replay()
         assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert gb.fp8_last_device_error() == 0
+
+
+# one cluster with 1, 2, 4 and 8 vectors a thread at their first and last
+# sizes, then the three-kernel form: flat and strided, rows shorter than a
+# warp's vectors, single elements, ragged ends; each alignment of x and q
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(1, 1), (1, 7), (7, 9), (256, 128), (257, 128), (4096, 8), (4097, 8), (128, 512),
+                                       (129, 512), (256, 512), (512, 512), (513, 512), (1, 262144), (1, 262145),
+                                       (32769, 3), (100000, 5), (5000, 100), (700, 1001), (64, 8200), (3, 200001)])
+def test_tensor_shapes(gb, orc, fmt, rows, cols):
+    x = workloads.randn_f32((rows, cols), seed=rows + 3 * cols)
+    x[-1, -1] = -77.0                                      # amax in the last element
+    qo, do = orc.quantize(x, 0, fmt=fmt)
+    quantize = gb.fp8_quantize_e5m2 if fmt else gb.fp8_quantize_e4m3
+    for pad, off, qpad, qoff in ((0, 0, 0, 0), (0, 4, 0, 4), (-cols % 8, 0, -cols % 16, 0), (1, 1, 3, 1),
+                                 (-cols % 4 + 4, 4, -cols % 4 + 4, 4)):
+        xb = torch.full((rows * (cols + pad) + off,), float("nan"), device="cuda")
+        xt = xb[off:].view(rows, cols + pad)[:, :cols]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((rows * (cols + qpad) + qoff,), 0xA5, dtype=torch.uint8, device="cuda")
+        qt = qb[qoff:].view(rows, cols + qpad)[:, :cols]
+        for _ in range(2):                                 # the scale slot holds the first pass's scale
+            _, d = quantize(xt, 0, q=qt)
+        assert np.array_equal(d.cpu().numpy(), do)
+        assert np.array_equal(qt.cpu().numpy(), qo)
+        if qpad:
+            assert bool((qb[qoff:].view(rows, cols + qpad)[:, cols:] == 0xA5).all())
+    torch.cuda.synchronize()
+    assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("rows,cols", [(64, 64), (700, 1001)])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_tensor_nonfinite_reported(gb, rows, cols, bad):
+    x = torch.randn((rows, cols), device="cuda")
+    x[rows - 1, cols - 2] = bad
+    gb.fp8_quantize_e4m3(x, 0)
+    assert gb.fp8_last_device_error() == -4
+    assert gb.fp8_last_device_error() == 0
