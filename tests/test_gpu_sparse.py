@@ -182,3 +182,32 @@ def test_sparse_extreme_shapes_small_integers_exact(gb, orc, M, N, K):
     assert np.array_equal(C.astype(np.float64), exact)
     ms, ns = workloads.sample_pairs(M, N, 256, seed=10)
     assert np.array_equal(C[ms, ns].astype(np.float64), orc.gemm_sampled(Ap, B, one, 0, one, 0, 1.0, ms, ns))
+
+
+@pytest.mark.parametrize("mt", [0, 1, 2, 3])
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("M,N", [(128, 16), (130, 15), (136, 17), (160, 33), (161, 64), (384, 100), (391, 129),
+                                 (1032, 300), (1027, 500), (2304, 250)])
+def test_transposed_output_edges(gb, mt, out, M, N):
+    """out_transposed with rows (M) and columns (N) that end inside tiles,
+    chunks and 16-byte pieces, aligned and unaligned row strides: exact
+    integers, nothing written outside the output."""
+    K = 256
+    A = torch.from_numpy(workloads.small_int_codes((M, K), seed=M, maxabs=2)).cuda()
+    B = torch.from_numpy(workloads.small_int_codes((N, K), seed=N, maxabs=2)).cuda()
+    v, m = gb.prune24_compress(A)
+    P = gb.prune24_decompress(v, m, K)
+    ref = (B.view(torch.float8_e4m3fn).double() @ P.view(torch.float8_e4m3fn).double().T).float()
+    one = torch.ones(1, device="cuda")
+    dt = torch.bfloat16 if out else torch.float32
+    gb.fp8_gemm_set_tile_config(mt, 0)
+    try:
+        for pad in (0, -M % 8, -M % 8 + 8, 1):
+            buf = torch.full((N + 1, M + pad), 7.0, dtype=dt, device="cuda")
+            C = buf[:N, :M]
+            gb.gemm_fp8_sparse24(v, m, B, one, 0, one, 0, out_dtype=out, out_transposed=True, C=C)
+            assert torch.equal(C.float(), ref.to(dt).float())
+            assert bool((buf[:N, M:] == 7).all()) and bool((buf[N] == 7).all())
+    finally:
+        gb.fp8_gemm_set_tile_config(0, 0)
+    assert gb.fp8_last_device_error() == 0
