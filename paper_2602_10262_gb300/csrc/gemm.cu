@@ -433,53 +433,56 @@ __device__ __forceinline__ void split_reduce_store(const ProblemScalars& P, cons
     }
 }
 
+// 16 accumulator columns of this thread's row, from tensor memory.
+__device__ __forceinline__ void tmem_sums16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    tmem_ld_32x32b_x16(taddr, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int t = 0; t < 16; ++t)
+        v[t] = __uint_as_float(r[t]);
+}
+
 // Split-K within a cluster (one unit per CTA, the slices of a tile as the
 // CTAs of one cluster, rank = slice).  Slice r > 0 writes its partial sums
-// into the idle TMA ring of the cluster's rank-0 CTA, column by column
-// (element (row, col) of slice r at ((r - 1) * bn + col) * rows_per_tile +
-// row floats from the ring's start).
-__device__ __forceinline__ void cluster_send_partial(const ProblemScalars& P, uint32_t leader_ring,
-                                                     int rows_per_tile, int slice, int row, uint32_t taddr,
-                                                     int c_lo, int c_hi)
+// into the rank-0 CTA's shared memory, column by column (element (row, col)
+// of slice r at ((r - 1) * bn + col) * rows_per_tile + row floats from `to`).
+// Where they fit beside the TMA ring (in the staging buffers, which a split
+// tile's epilogue does not use) they are sent at once; else into the ring,
+// once the rank-0 CTA has said that its MMAs are done with it.  That
+// handshake, a cluster barrier at the end and the lane-by-lane stores of the
+// sum took longer than the k-loop of 16 x 4096 x 4096 (3.6 against 1.5 us):
+// with its quantise that launch takes 9.2 us, 10.4 before, 64 x 8192 x 8192
+// 17.1 (19.1), 2:4 64 x 8192 x 8192 14.0 (16.0).
+__device__ __forceinline__ void cluster_send_partial(const ProblemScalars& P, uint32_t to, int rows_per_tile,
+                                                     int slice, int row, uint32_t taddr, int c_lo, int c_hi)
 {
-    const uint32_t base = leader_ring + 4u * static_cast<uint32_t>((slice - 1) * P.bn * rows_per_tile + row);
+    const uint32_t base = to + 4u * static_cast<uint32_t>((slice - 1) * P.bn * rows_per_tile + row);
     for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(taddr + c0, r);
-        tmem_ld_wait();
+        float v[16];
+        tmem_sums16(taddr + c0, v);
 #pragma unroll
         for (int t = 0; t < 16; ++t)
-            st_cluster_f32(base + 4u * static_cast<uint32_t>((c0 + t) * rows_per_tile), __uint_as_float(r[t]));
+            st_cluster_f32(base + 4u * static_cast<uint32_t>((c0 + t) * rows_per_tile), v[t]);
     }
 }
 
-// The rank-0 CTA: its own partial from TMEM, then the other slices' from its
-// ring, added in slice order (the same sums as the global split path), then
-// scaled and stored.
-__device__ __forceinline__ void cluster_reduce_store(const ProblemScalars& P, const uint8_t* ring,
-                                                     int rows_per_tile, int row, uint32_t taddr, int i,
-                                                     bool row_ok, float fi, int jbase, ScaleWindows& sw,
-                                                     int lane, int c_lo, int c_hi)
+// The rank-0 CTA's sums of 16 columns: its own partial from tensor memory,
+// then the other slices' from `recv` (this row's first float), added in slice
+// order (the same sums as the global split path).
+__device__ __forceinline__ void cluster_sums16(const ProblemScalars& P, const float* recv, int rows_per_tile,
+                                               uint32_t taddr, int c, float (&acc)[16])
 {
-    const float* recv = reinterpret_cast<const float*>(ring) + row;
-    float s_cur = 0.0f;
-    for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-        if ((c0 & 31) == 0)
-            s_cur = sw.take(P, jbase + c_lo, lane);
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(taddr + c0, r);
-        tmem_ld_wait();
-        float acc[16];
+    tmem_sums16(taddr + c, acc);
+#pragma unroll
+    for (int t = 0; t < 16; ++t)
+        acc[t] = __fadd_rn(0.0f, acc[t]);
+    for (int sl = 1; sl < P.splits; ++sl) {
+        const float* col = recv + ((sl - 1) * P.bn + c) * rows_per_tile;
 #pragma unroll
         for (int t = 0; t < 16; ++t)
-            acc[t] = __fadd_rn(0.0f, __uint_as_float(r[t]));
-        for (int sl = 1; sl < P.splits; ++sl) {
-            const float* col = recv + ((sl - 1) * P.bn + c0) * rows_per_tile;
-#pragma unroll
-            for (int t = 0; t < 16; ++t)
-                acc[t] = __fadd_rn(acc[t], col[t * rows_per_tile]);
-        }
-        store_vals16(P, i, row_ok, fi, jbase + c0, acc, s_cur, c0 & 31);
+            acc[t] = __fadd_rn(acc[t], col[t * rows_per_tile]);
     }
 }
 
@@ -683,8 +686,9 @@ __device__ __forceinline__ void epilogue_rows_coalesced(const ProblemScalars& P,
 // 2:4 128 x 8192 x 8192 were that epilogue.  That product takes 16.2 us now,
 // 4096 x 14336 x 4096 119 (127), dense 128 x 8192 x 8192 20.0 (23.1).  A
 // partial last chunk (narrower than the box) is stored by the lanes.
-template <int ESZ, int NB>
-__device__ __forceinline__ void epilogue_cols_staged(const ProblemScalars& P, uint32_t taddr, int i, bool row_ok,
+// load(c, acc): the 16 sums of columns c .. c + 15 of this lane's row.
+template <int ESZ, int NB, typename Load>
+__device__ __forceinline__ void epilogue_cols_staged(const ProblemScalars& P, Load load, int i, bool row_ok,
                                                      float fi, int jbase, uint8_t* bufs, int lane, ScaleWindows& sw,
                                                      const CUtensorMap* tmC, int c_lo, int c_hi)
 {
@@ -708,17 +712,16 @@ __device__ __forceinline__ void epilogue_cols_staged(const ProblemScalars& P, ui
         for (int q = 0; q < cw; q += 16) {
             if (((c0 + q - c_lo) & 31) == 0)
                 s_cur = sw.take(P, jbase + c_lo, lane);
-            uint32_t r[16];
-            tmem_ld_32x32b_x16(taddr + c0 + q, r);
-            tmem_ld_wait();
+            float acc[16];
+            load(c0 + q, acc);
             if (cw < CW) {
-                store_chunk16(P, i, row_ok, fi, jbase + c0 + q, r, s_cur, (c0 + q - c_lo) & 31);
+                store_vals16(P, i, row_ok, fi, jbase + c0 + q, acc, s_cur, (c0 + q - c_lo) & 31);
                 continue;
             }
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
                 const float sj = __shfl_sync(0xFFFFFFFFu, s_cur, ((c0 + q - c_lo) & 31) + t);
-                const float v = __fmul_rn(__fmul_rn(__uint_as_float(r[t]), fi), sj);
+                const float v = __fmul_rn(__fmul_rn(acc[t], fi), sj);
                 if (ESZ == 2)
                     reinterpret_cast<__nv_bfloat16*>(buf)[(q + t) * 32 + lane] = __float2bfloat16_rn(v);
                 else
@@ -786,7 +789,9 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     // and the asm statements below would otherwise make the compiler repeat
     // them on the critical path).
     const int total_tiles = prm.total_tiles;
-    const int cluster_split = prm.cluster_split;
+    // (only one-problem launches add slices up within clusters)
+    constexpr bool kCanSplitCluster = MAXP == 1 && !PAIR && MX == 0;
+    const int cluster_split = kCanSplitCluster ? prm.cluster_split : 0;
     int* const err = prm.err;
     const unsigned long long wlim = prm.wait_ns;
     float* const ws = prm.ws;
@@ -895,14 +900,20 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
         }
     }
     // Q multicast: every CTA's barriers exist before a peer's copies or
-    // commits reach them
+    // commits reach them.  Cluster split-K: the same before a partial sum is
+    // sent; the wait for it comes when one is, or at the end.
     if (!PAIR && mc > 0)
         cluster_sync();
-    // Everything above reads only the kernel parameters and shared memory;
-    // from here on the previous kernel's outputs (operands, scales, the
-    // split-K workspace) are read and written.
-    grid_dependency_wait();
+    if (cluster_split)
+        cluster_arrive();
+    // Everything above reads only the kernel parameters and shared memory.
+    // The previous kernel's outputs (operands, scales, the split-K workspace)
+    // are read and written by the producer and the epilogue, each of which
+    // waits for that kernel itself, the producer with its first stage armed
+    // and its first load the next instruction; the MMA warp reads what the
+    // producer loaded.
 
+    bool cluster_waited = false;                // this thread has waited for the first cluster barrier
     // Roles are chosen per warp; inside warps 0 and 1 only lane 0 works.
     if (warp == 0) {
         if (lane == 0) {
@@ -915,6 +926,12 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             // pairs: the even CTA arms its "full" barrier for both CTAs' bytes
             // and both CTAs' loads complete on it
             const uint32_t full_rank = PAIR ? 0u : rank;
+            bool waited = false;
+            const auto previous_kernel_done = [&] {
+                if (!waited)
+                    grid_dependency_wait();
+                waited = true;
+            };
             for (int tile = tile0; ok && tile < producer_tiles; tile += tile_step) {
                 const TileCoord tc = tile == tile0 ? tc_first : tile_coord(prm, tile);
                 const bool first = tile == tile0;
@@ -962,6 +979,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                             mbar_arrive_expect_tx(fb, 2u * (static_cast<uint32_t>(C::kAChunk) + b_chunk) *
                                                               static_cast<uint32_t>(P.tma3d ? KC : nck) +
                                                           (MX ? 2u * (1 + C::kSfQ) * KC * C::kSfChunk : 0u));
+                        previous_kernel_done();
                         if constexpr (MX) {
                             const uint32_t sf = sa + C::kABytes + C::kBBytes;
                             tma_load_3d_pair(sf, &prm.prob[tc.p].tmE, fb, 0, kb,
@@ -1008,6 +1026,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                     mbar_arrive_expect_tx(full_bar(stage),
                                           a_bytes * p_chunks + b_chunk * q_chunks +
                                               sf_chunks * C::kSfChunk * static_cast<uint32_t>(nck));
+                    previous_kernel_done();
                     if (sparse && KC > 1) {
                         // kept codes then metadata of all KC k-blocks (3-D chunk boxes)
                         tma_load_3d(sa, map_p, full_bar(stage), 0, row0, kb);
@@ -1302,6 +1321,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
         const int row = half * BM + quarter * 32 + lane;
         int local = 0;
         uint32_t split_phase = 0;
+        grid_dependency_wait();
         for (int tile = tile0; tile < my_tiles; tile += tile_step, ++local) {
             const TileCoord tc = tile == tile0 ? tc_first : tile_coord(prm, tile);
             const ProblemScalars P = tile == tile0 ? P_first : prm.prob[tc.p];
@@ -1344,15 +1364,21 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
                                    static_cast<uint32_t>(acc * C::kAcc1 + half * BN_MAX);
-            if (P.splits > 1 && cluster_split) {
+            if (kCanSplitCluster && P.splits > 1 && cluster_split) {
                 const int crank = static_cast<int>(cluster_ctarank());
                 if (crank != tc.slice) {                // launch shape broken: never expected
                     abort_pipeline(abort_flag, err);
                     break;
                 }
+                const int rows_per_tile = BM * MT;
+                const bool beside = (P.splits - 1) * P.bn * rows_per_tile * 4 <= C::kEpiBytes;
+                uint8_t* recv = beside ? epi_smem : smem;
+                if (!cluster_waited)
+                    cluster_wait();                     // every CTA of the cluster is up
+                cluster_waited = true;
                 if (crank == 0) {
                     // every MMA of this unit has completed: the ring is free
-                    if (threadIdx.x == 64)
+                    if (!beside && threadIdx.x == 64)
                         for (int r = 1; r < P.splits; ++r)
                             mbar_arrive_remote(cluster_map(split_verdict_bar, static_cast<uint32_t>(r)));
                     const bool got = mbar_wait_cluster(split_written_bar, 0u, abort_flag, wlim);
@@ -1360,14 +1386,41 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                         abort_pipeline(abort_flag, err);
                         break;
                     }
-                    cluster_reduce_store(P, smem, BM * MT, row, taddr, i, row_ok, fi, jbase, sw, lane, c_lo, c_hi);
+                    const float* mine = reinterpret_cast<const float*>(recv) + row;
+                    const auto load = [&](int c, float (&v)[16]) {
+                        cluster_sums16(P, mine, rows_per_tile, taddr, c, v);
+                    };
+                    // staging buffers: whichever of the two regions the
+                    // partial sums are not in
+                    uint8_t* stage_buf = (beside ? smem : epi_smem) + (warp - 2) * 32 * 128;
+                    const int first_row = i - lane;
+                    if (P.trans_out && P.tma_store &&
+                        (first_row + 32 <= P.rows_p || P.rows_p * (P.out_bf16 ? 2 : 4) % 16 == 0)) {
+                        const CUtensorMap* map_c = &prm.prob[tc.p].tmC;
+                        if (P.out_bf16)
+                            epilogue_cols_staged<2, 1>(P, load, i, row_ok, fi, jbase, stage_buf, lane, sw, map_c, c_lo,
+                                                       c_hi);
+                        else
+                            epilogue_cols_staged<4, 1>(P, load, i, row_ok, fi, jbase, stage_buf, lane, sw, map_c, c_lo,
+                                                       c_hi);
+                    } else {
+                        float s_cur = 0.0f;
+                        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+                            if (((c0 - c_lo) & 31) == 0)
+                                s_cur = sw.take(P, jbase + c_lo, lane);
+                            float v[16];
+                            load(c0, v);
+                            store_vals16(P, i, row_ok, fi, jbase + c0, v, s_cur, (c0 - c_lo) & 31);
+                        }
+                    }
                 } else {
-                    const bool got = mbar_wait_cluster(split_verdict_bar, 0u, abort_flag, wlim);
+                    const bool got = beside || mbar_wait_cluster(split_verdict_bar, 0u, abort_flag, wlim);
                     if (!__all_sync(0xFFFFFFFFu, got)) {
                         abort_pipeline(abort_flag, err);
                         break;
                     }
-                    cluster_send_partial(P, cluster_map(smem_base, 0u), BM * MT, crank, row, taddr, c_lo, c_hi);
+                    cluster_send_partial(P, cluster_map(smem_u32(recv), 0u), rows_per_tile, crank, row, taddr, c_lo,
+                                         c_hi);
                     mbar_arrive_remote(cluster_map(split_written_bar, 0u));
                 }
                 tc_fence_before();
@@ -1461,11 +1514,12 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             } else if (tmC != nullptr && (row0 + 32 <= P.rows_p || P.rows_p * (P.out_bf16 ? 2 : 4) % 16 == 0)) {
                 // (a warp whose rows end inside a 16-byte piece stores them
                 // itself, as does a warp with no rows: TMA clips to 16 bytes)
+                const auto load = [&](int c, float (&v)[16]) { tmem_sums16(taddr + c, v); };
                 if (P.out_bf16)
-                    epilogue_cols_staged<2, C::kEpiBufs>(P, taddr, i, row_ok, fi, jbase, buf, lane, sw, tmC, c_lo,
+                    epilogue_cols_staged<2, C::kEpiBufs>(P, load, i, row_ok, fi, jbase, buf, lane, sw, tmC, c_lo,
                                                         c_hi);
                 else
-                    epilogue_cols_staged<4, C::kEpiBufs>(P, taddr, i, row_ok, fi, jbase, buf, lane, sw, tmC, c_lo,
+                    epilogue_cols_staged<4, C::kEpiBufs>(P, load, i, row_ok, fi, jbase, buf, lane, sw, tmC, c_lo,
                                                         c_hi);
             } else {
                 float s_cur = 0.0f;
@@ -1489,14 +1543,22 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     // In warps 0 and 1 only lane 0 ran a role loop: reconverge every warp
     // before the CTA-wide barrier (bar.sync is warp-aligned).
     __syncwarp();
+    if (cluster_split && !cluster_waited)
+        cluster_wait();
     tc_fence_before();
     __syncthreads();
-    // cluster split-K: no CTA leaves while a peer may still write to its
-    // shared memory; pairs: neither CTA frees the pair's tensor memory (or
-    // its barriers) while the other may still use them (every wait above is
-    // bounded, so all threads get here)
-    if (PAIR || cluster_split || mc > 0)
+    // cluster split-K: the rank-0 CTA does not leave while a peer may still
+    // write to its shared memory (nobody writes to the others', which signal
+    // and go); pairs and multicast: neither CTA frees the pair's tensor memory
+    // (or its barriers) while the other may still use them (every wait above
+    // is bounded, so all threads get here)
+    if (cluster_split) {
+        cluster_arrive();
+        if (cluster_ctarank() == 0)
+            cluster_wait();
+    } else if (PAIR || mc > 0) {
         cluster_sync();
+    }
     if (warp == 1) {
         tc_fence_after();
         if constexpr (PAIR)

@@ -418,3 +418,33 @@ def test_rows_that_start_anywhere(gb, mt, out, M, N, K):
     finally:
         gb.fp8_gemm_set_tile_config(0, 0)
     assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("sparse", [False, True])
+@pytest.mark.parametrize("rows,N,K", [(1, 520, 4096), (16, 1029, 4224), (17, 4096, 4096), (33, 2050, 8192),
+                                      (64, 1544, 8192), (64, 8192, 8192), (100, 777, 8192), (128, 128, 16384)])
+def test_split_clusters_exact(gb, out, sparse, rows, N, K):
+    """Products split along K within clusters, partial sums beside the ring
+    and in it, outputs that end inside tiles and 16-byte pieces: integers
+    exact, columns past the output untouched."""
+    W = _cuda(workloads.small_int_codes((N, K), seed=N, maxabs=2))
+    X = _cuda(workloads.small_int_codes((rows, K), seed=rows, maxabs=2))
+    plan = gb.gemm_fp8_sparse24_plan(N, rows, K, out) if sparse else gb.gemm_fp8_dense_plan(rows, N, K, out)
+    assert plan["splits"] > 1, plan
+    if sparse:
+        v, m = gb.prune24_compress(W)
+        W = gb.prune24_decompress(v, m, K)
+    ref = (X.view(torch.float8_e4m3fn).double() @ W.view(torch.float8_e4m3fn).double().T).float()
+    dt = torch.bfloat16 if out else torch.float32
+    for pad in (0, -N % 8 + 8, 1):
+        buf = torch.full((rows + 1, N + pad), 7.0, dtype=dt, device="cuda")
+        C = buf[:rows, :N]
+        for _ in range(3):
+            if sparse:
+                gb.gemm_fp8_sparse24(v, m, X, _ones(), 0, _ones(), 0, out_dtype=out, out_transposed=True, C=C)
+            else:
+                gb.gemm_fp8_dense(X, W, _ones(), 0, _ones(), 0, 1.0, out, C=C)
+        assert torch.equal(C.float(), ref.to(dt).float())
+        assert bool((buf[:rows, N:] == 7).all()) and bool((buf[rows] == 7).all())
+    assert gb.fp8_last_device_error() == 0
