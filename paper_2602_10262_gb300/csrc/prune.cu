@@ -4,7 +4,7 @@
 // codes): one 16-byte load, a branch-free selection for the four groups at
 // once (select_groups4), an 8-byte store of the kept codes and a 2-byte
 // store of the four metadata nibbles.  Rows whose length or alignment does
-// not allow it fall back to one metadata byte per iteration.
+// not allow it take the same pieces with narrower accesses.
 // Bandwidth-bound: 1 byte read, 0.625 bytes written per element; no
 // allocation, one launch.  The inverse moves the same bytes the other way.
 #include <algorithm>
@@ -22,8 +22,8 @@ constexpr int kThreads = 256;
 // 16 codes (four groups) spaced kThreads apart, so each load instruction of
 // a warp reads 512 contiguous bytes; all loads are issued before any
 // selection.  Per piece: 8 bytes of kept codes and 16 bits of metadata.
-// Contiguous rows (lda == K) come as one long row, so every block but the
-// last has all its pieces whatever K is: a block per row of K = 8192 has
+// Contiguous rows (lda == K, K % 8 == 0) come as one long row, so every block
+// but the last has all its pieces whatever K is: a block per row of K = 8192 has
 // work for half of its loads, one of K = 1024 for a sixteenth.  Measured
 // (GB300, inputs rotated beyond L2) with both changes, the four-group
 // selection and the one long row: 23.3 -> 17.3 us at 8192 x 8192 (6.3 TB/s),
@@ -70,39 +70,140 @@ __global__ void __launch_bounds__(kThreads) prune24_vec_kernel(const uint8_t* __
     }
 }
 
-// Scalar path (any K % 4 == 0 and any alignment): one metadata byte (two
-// groups, or one at an odd tail) per iteration so that no two threads write
-// the same byte.
-__global__ void __launch_bounds__(kThreads) prune24_kernel(const uint8_t* __restrict__ a,
-                                                           int64_t M, int64_t K, int64_t lda,
-                                                           uint8_t* __restrict__ vals,
-                                                           uint8_t* __restrict__ meta)
+// Any K % 4 == 0 and any alignment: a row is ceil(K / 16) pieces of up to
+// four groups, and a thread takes U pieces of the whole matrix (kThreads
+// apart, the row by one 32-bit division), each with the widest loads and
+// stores its arrays allow.  16384 x 4100 (rows of half metadata bytes): 28.6
+// us, and 46.2 to expand it again; one metadata byte, or one group, per
+// thread with single-byte accesses and a 64-bit division took 46.8 and 54.9.
+struct PieceShape {
+    int64_t total;             // pieces of the matrix
+    int64_t per_row;
+    int64_t groups;            // of a row
+    int64_t ldv, ldm;          // kept-code and metadata bytes of a row
+};
+
+__device__ __forceinline__ void piece_row(const PieceShape& s, int64_t i, int64_t* r, int64_t* p)
+{
+    if (s.total <= 0xFFFFFFFFll) {
+        const uint32_t n = static_cast<uint32_t>(s.per_row);
+        const uint32_t q = static_cast<uint32_t>(i) / n;
+        *r = q;
+        *p = static_cast<uint32_t>(i) - q * n;
+    } else {
+        *r = i / s.per_row;
+        *p = i - *r * s.per_row;
+    }
+}
+
+// n bytes (a multiple of 2, at most 4 * W) between memory of alignment
+// `align` (16, 8, 4, 2 or 1) and words.
+template <int W>
+__device__ __forceinline__ void load_words(const uint8_t* p, int n, int align, uint32_t (&w)[W])
+{
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+        w[i] = 0;
+    if (W == 4 && align >= 16 && n == 16) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+        w[0] = v.x, w[W > 1 ? 1 : 0] = v.y, w[W > 2 ? 2 : 0] = v.z, w[W > 3 ? 3 : 0] = v.w;
+    } else if (W >= 2 && align >= 8 && n == 4 * W) {
+#pragma unroll
+        for (int i = 0; i + 1 < W; i += 2) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + 4 * i));
+            w[i] = v.x, w[i + 1] = v.y;
+        }
+    } else if (align >= 4) {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (4 * i + 4 <= n)
+                w[i] = __ldg(reinterpret_cast<const uint32_t*>(p + 4 * i));
+            else if (4 * i + 2 <= n)
+                w[i] = __ldg(reinterpret_cast<const uint16_t*>(p + 4 * i));
+    } else if (align >= 2) {
+#pragma unroll
+        for (int i = 0; i < 2 * W; ++i)
+            if (2 * i + 2 <= n)
+                w[i / 2] |= static_cast<uint32_t>(__ldg(reinterpret_cast<const uint16_t*>(p + 2 * i))) << (16 * (i & 1));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4 * W; ++i)
+            if (i < n)
+                w[i / 4] |= static_cast<uint32_t>(__ldg(p + i)) << (8 * (i & 3));
+    }
+}
+
+template <int W>
+__device__ __forceinline__ void store_words(uint8_t* p, int n, int align, const uint32_t (&w)[W])
+{
+    if (W >= 2 && align >= 8 && n == 4 * W) {
+#pragma unroll
+        for (int i = 0; i + 1 < W; i += 2)
+            *reinterpret_cast<uint2*>(p + 4 * i) = make_uint2(w[i], w[i + 1]);
+    } else if (align >= 4) {
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (4 * i + 4 <= n)
+                *reinterpret_cast<uint32_t*>(p + 4 * i) = w[i];
+            else if (4 * i + 2 <= n)
+                *reinterpret_cast<uint16_t*>(p + 4 * i) = static_cast<uint16_t>(w[i]);
+    } else if (align >= 2) {
+#pragma unroll
+        for (int i = 0; i < 2 * W; ++i)
+            if (2 * i + 2 <= n)
+                *reinterpret_cast<uint16_t*>(p + 2 * i) = static_cast<uint16_t>(w[i / 2] >> (16 * (i & 1)));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4 * W; ++i)
+            if (i < n)
+                p[i] = static_cast<uint8_t>(w[i / 4] >> (8 * (i & 3)));
+    }
+}
+
+template <int U>
+__global__ void __launch_bounds__(kThreads) prune24_any_kernel(const uint8_t* __restrict__ a, PieceShape s,
+                                                               int64_t lda, int a_align, uint8_t* __restrict__ vals,
+                                                               int v_align, uint8_t* __restrict__ meta, int m_align)
 {
     grid_launch_dependents();
     grid_dependency_wait();
-    const int64_t ldv = K / 2, ldm = (K + 7) / 8;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
-    const int64_t tid = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x;
-    for (int64_t i = tid; i < M * ldm; i += stride) {
-        const int64_t r = i / ldm, b = i - r * ldm;
-        uint8_t out = 0;
-        for (int h = 0; h < 2; ++h) {
-            const int64_t g = 2 * b + h;
-            if (4 * g >= K)
-                break;
-            const uint8_t* p = a + r * lda + 4 * g;
-            const uint32_t w = p[0] | (p[1] << 8) | (p[2] << 16) | (static_cast<uint32_t>(p[3]) << 24);
-            const uint32_t sel = select_group(w);
-            vals[r * ldv + 2 * g] = static_cast<uint8_t>(sel & 0xFFu);
-            vals[r * ldv + 2 * g + 1] = static_cast<uint8_t>((sel >> 8) & 0xFFu);
-            out |= static_cast<uint8_t>(((sel >> 16) & 0xFu) << (4 * h));
+    const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads * U);
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kThreads * U) + threadIdx.x; i0 < s.total; i0 += step) {
+        uint32_t w[U][4];
+        int64_t r[U], p[U];
+        int n[U];                          // groups of the piece
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * kThreads;
+            n[u] = 0;
+            if (i < s.total) {
+                piece_row(s, i, &r[u], &p[u]);
+                n[u] = static_cast<int>(min(static_cast<int64_t>(4), s.groups - 4 * p[u]));
+                load_words<4>(a + r[u] * lda + 16 * p[u], 4 * n[u], a_align, w[u]);
+            }
         }
-        meta[r * ldm + b] = out;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (n[u] == 0)
+                continue;
+            uint32_t v[2];
+            const uint32_t nib =
+                select_groups4(w[u][0], w[u][1], w[u][2], w[u][3], &v[0], &v[1]) & ((1u << (4 * n[u])) - 1u);
+            store_words<2>(vals + r[u] * s.ldv + 8 * p[u], 2 * n[u], v_align, v);
+            uint8_t* md = meta + r[u] * s.ldm + 2 * p[u];
+            if (m_align >= 2 && n[u] > 2) {
+                *reinterpret_cast<uint16_t*>(md) = static_cast<uint16_t>(nib);
+            } else {
+                md[0] = static_cast<uint8_t>(nib);
+                if (n[u] > 2)
+                    md[1] = static_cast<uint8_t>(nib >> 8);
+            }
+        }
     }
 }
 
 // One group expanded: the two kept codes of v's low half at the bytes the
-// nibble names (any nibble, equal indices included, as the scalar path).
+// nibble names (any nibble: equal or descending indices combine with OR).
 __device__ __forceinline__ uint32_t expand_group(uint32_t v, uint32_t nib)
 {
     return ((v & 0xFFu) << ((nib << 3) & 24u)) | (((v >> 8) & 0xFFu) << ((nib << 1) & 24u));
@@ -113,8 +214,8 @@ __device__ __forceinline__ uint32_t expand_group(uint32_t v, uint32_t nib)
 // of pieces (8 kept codes and 16 metadata bits -> 16 codes); a thread takes
 // U of them (pieces_per_thread) spaced kThreads apart, all loads before any
 // store.  Bound by HBM: 18.0 us at 8192 x 8192 (6.1 TB/s), 64.3 us at 16384 x
-// 16384, against 56.1 and 212 us for the scalar path below (single-byte
-// loads and stores, a 64-bit division per group).
+// 16384, against 56.1 and 212 us with single-byte loads and stores and a
+// 64-bit division per group.
 template <int U>
 __global__ void __launch_bounds__(kThreads) decompress24_vec_kernel(const uint2* __restrict__ vals,
                                                                     const uint16_t* __restrict__ meta,
@@ -145,37 +246,65 @@ __global__ void __launch_bounds__(kThreads) decompress24_vec_kernel(const uint2*
     }
 }
 
-// Scalar path (any K % 4 == 0 and any alignment): one group per iteration.
-__global__ void __launch_bounds__(kThreads) decompress24_kernel(const uint8_t* __restrict__ vals,
-                                                                const uint8_t* __restrict__ meta,
-                                                                int64_t M, int64_t K,
-                                                                uint8_t* __restrict__ out)
+// The inverse for any K % 4 == 0 and any alignment, by the same pieces.
+template <int U>
+__global__ void __launch_bounds__(kThreads) decompress24_any_kernel(const uint8_t* __restrict__ vals, int v_align,
+                                                                    const uint8_t* __restrict__ meta, int m_align,
+                                                                    PieceShape s, uint8_t* __restrict__ out,
+                                                                    int64_t ldo, int o_align)
 {
     grid_launch_dependents();
     grid_dependency_wait();
-    const int64_t ldv = K / 2, ldm = (K + 7) / 8, groups = K / 4;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < M * groups;
-         i += stride) {
-        const int64_t r = i / groups, g = i - r * groups;
-        const uint32_t nib = (meta[r * ldm + g / 2] >> (4 * (g % 2))) & 0xFu;
-        const uint32_t i0 = nib & 3u, i1 = nib >> 2;
-        uint32_t w = 0;
-        w |= static_cast<uint32_t>(vals[r * ldv + 2 * g]) << (8 * i0);
-        w |= static_cast<uint32_t>(vals[r * ldv + 2 * g + 1]) << (8 * i1);
-        uint8_t* o = out + r * K + 4 * g;
-        o[0] = w & 0xFFu;
-        o[1] = (w >> 8) & 0xFFu;
-        o[2] = (w >> 16) & 0xFFu;
-        o[3] = (w >> 24) & 0xFFu;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads * U);
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kThreads * U) + threadIdx.x; i0 < s.total; i0 += step) {
+        uint32_t v[U][2], m[U];
+        int64_t r[U], p[U];
+        int n[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * kThreads;
+            n[u] = 0;
+            if (i < s.total) {
+                piece_row(s, i, &r[u], &p[u]);
+                n[u] = static_cast<int>(min(static_cast<int64_t>(4), s.groups - 4 * p[u]));
+                load_words<2>(vals + r[u] * s.ldv + 8 * p[u], 2 * n[u], v_align, v[u]);
+                const uint8_t* md = meta + r[u] * s.ldm + 2 * p[u];
+                if (m_align >= 2 && n[u] > 2) {
+                    m[u] = __ldg(reinterpret_cast<const uint16_t*>(md));
+                } else {
+                    m[u] = __ldg(md);
+                    if (n[u] > 2)
+                        m[u] |= static_cast<uint32_t>(__ldg(md + 1)) << 8;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (n[u] == 0)
+                continue;
+            const uint32_t w[4] = {expand_group(v[u][0], m[u]), expand_group(v[u][0] >> 16, m[u] >> 4),
+                                   expand_group(v[u][1], m[u] >> 8), expand_group(v[u][1] >> 16, m[u] >> 12)};
+            store_words<4>(out + r[u] * ldo + 16 * p[u], 4 * n[u], o_align, w);
+        }
     }
 }
 
-int grid_for(int64_t items)
+// The largest of 16, 8, 4, 2, 1 that divides a base address and a row stride.
+int bytes_align(const void* p, int64_t ld)
 {
-    const int64_t blocks = (items + kThreads - 1) / kThreads;
-    const int64_t cap = static_cast<int64_t>(sm_count()) * 16;
-    return static_cast<int>(blocks < cap ? (blocks > 0 ? blocks : 1) : cap);
+    const uint64_t v = reinterpret_cast<uintptr_t>(p) | static_cast<uint64_t>(ld) | 16;
+    return static_cast<int>(v & (~v + 1));
+}
+
+PieceShape piece_shape(int64_t M, int64_t K)
+{
+    const int64_t per_row = (K + 15) / 16;
+    return {M * per_row, per_row, K / 4, K / 2, (K + 7) / 8};
+}
+
+unsigned piece_grid(int64_t total, int u)
+{
+    return static_cast<unsigned>(std::min<int64_t>((total + kThreads * u - 1) / (kThreads * u), INT32_MAX));
 }
 
 }  // namespace
@@ -198,16 +327,18 @@ extern "C" int prune24_compress(const uint8_t* a, int64_t M, int64_t K, int64_t 
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const bool vec = (K % 16 == 0) && aligned16(a) && (lda % 16 == 0) &&
+    // contiguous rows of whole metadata bytes are one row (the vector path's
+    // piece index is 32 bits)
+    if (lda == K && K % 8 == 0 && M * (K / 8) < INT32_MAX) {
+        K *= M;
+        lda = K;
+        M = 1;
+    }
+    const int64_t row_a = M == 1 ? 0 : lda;       // one row: its start alone decides the alignment
+    const bool vec = (K % 16 == 0) && aligned16(a) && (row_a % 16 == 0) && K / 16 < INT32_MAX - kThreads * kPieces &&
                      (reinterpret_cast<uintptr_t>(a_vals) % 8 == 0) &&
                      (reinterpret_cast<uintptr_t>(a_meta) % 2 == 0);
     if (vec) {
-        // contiguous rows as one (the piece index of a row is 32 bits)
-        if (lda == K && M * (K / 16) < INT32_MAX - kThreads * kPieces) {
-            K *= M;
-            lda = K;
-            M = 1;
-        }
         const int64_t pieces = K / 16;
         const int u = pieces_per_thread(M * pieces);
         const unsigned gx = static_cast<unsigned>((pieces + kThreads * u - 1) / (kThreads * u));
@@ -217,7 +348,12 @@ extern "C" int prune24_compress(const uint8_t* a, int64_t M, int64_t K, int64_t 
         else
             launch_dependent(prune24_vec_kernel<kPieces>, dim3(gx, gy), kThreads, st, a, M, K, lda, a_vals, a_meta);
     } else {
-        launch_dependent(prune24_kernel, grid_for(M * ((K + 7) / 8)), kThreads, st, a, M, K, lda, a_vals, a_meta);
+        const PieceShape s = piece_shape(M, K);
+        const int u = pieces_per_thread(s.total);
+        const int aa = bytes_align(a, row_a), va = bytes_align(a_vals, M == 1 ? 0 : s.ldv),
+                  ma = bytes_align(a_meta, M == 1 ? 0 : s.ldm);
+        launch_dependent(u == 1 ? prune24_any_kernel<1> : prune24_any_kernel<kPieces>, piece_grid(s.total, u),
+                         kThreads, st, a, s, lda, aa, a_vals, va, a_meta, ma);
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
@@ -238,6 +374,10 @@ extern "C" int prune24_decompress(const uint8_t* a_vals, const uint8_t* a_meta, 
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (K % 8 == 0) {                             // rows of whole metadata bytes: one row
+        K *= M;
+        M = 1;
+    }
     if (K % 16 == 0 && aligned16(out) && reinterpret_cast<uintptr_t>(a_vals) % 8 == 0 &&
         reinterpret_cast<uintptr_t>(a_meta) % 2 == 0) {
         const int64_t pieces = M * (K / 16);
@@ -247,11 +387,18 @@ extern "C" int prune24_decompress(const uint8_t* a_vals, const uint8_t* a_meta, 
         const auto* m2 = reinterpret_cast<const uint16_t*>(a_meta);
         auto* o16 = reinterpret_cast<uint4*>(out);
         if (u == 1)
-            launch_dependent(decompress24_vec_kernel<1>, static_cast<unsigned>(blocks), kThreads, st, v8, m2, pieces, o16);
+            launch_dependent(decompress24_vec_kernel<1>, static_cast<unsigned>(blocks), kThreads, st, v8, m2, pieces,
+                             o16);
         else
-            launch_dependent(decompress24_vec_kernel<kPieces>, static_cast<unsigned>(blocks), kThreads, st, v8, m2, pieces, o16);
+            launch_dependent(decompress24_vec_kernel<kPieces>, static_cast<unsigned>(blocks), kThreads, st, v8, m2,
+                             pieces, o16);
     } else {
-        launch_dependent(decompress24_kernel, grid_for(M * (K / 4)), kThreads, st, a_vals, a_meta, M, K, out);
+        const PieceShape s = piece_shape(M, K);
+        const int u = pieces_per_thread(s.total);
+        const int va = bytes_align(a_vals, M == 1 ? 0 : s.ldv), ma = bytes_align(a_meta, M == 1 ? 0 : s.ldm),
+                  oa = bytes_align(out, M == 1 ? 0 : K);
+        launch_dependent(u == 1 ? decompress24_any_kernel<1> : decompress24_any_kernel<kPieces>,
+                         piece_grid(s.total, u), kThreads, st, a_vals, va, a_meta, ma, s, out, K, oa);
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;

@@ -64,7 +64,9 @@ def test_bad_k(gb):
 
 
 @pytest.mark.parametrize("M,K,pad", [(1, 16, 0), (3, 16, 0), (1025, 16, 0), (7, 1024, 0), (5, 1040, 16),
-                                     (2, 16400, 0), (33, 4096, 32), (6, 24, 0), (6, 24, 8), (4, 1028, 0)])
+                                     (2, 16400, 0), (33, 4096, 32), (6, 24, 0), (6, 24, 8), (4, 1028, 0), (1, 4, 0),
+                                     (5, 4, 4), (9, 12, 0), (9, 20, 12), (300, 1032, 0), (301, 1036, 4), (64, 8, 8),
+                                     (2100, 132, 0), (3, 4100, 3), (1, 40, 0)])
 def test_contiguous_and_strided_rows(orc, M, K, pad):
     """Rows as one run of 16-code pieces (lda == K), row by row (padded
     rows) and the scalar path (K % 16 != 0), at the edges of a block's 1024
