@@ -255,13 +255,27 @@ template <int FMT, int TPR, int U, int W>
 __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float* __restrict__ x, int64_t rows,
                                                                      int64_t cols, int64_t ldx,
                                                                      uint8_t* __restrict__ q, int64_t ldq,
-                                                                     float* __restrict__ d, int vec, int qa, int* err)
+                                                                     float* __restrict__ d, int vec, int qa,
+                                                                     int early, int* err)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     __shared__ uint32_t red[2][32];
     constexpr int kRows = row_block<TPR>() / TPR;         // rows per block
     const int t = threadIdx.x % TPR;
+    if (early) {
+        // the row into L2 while the previous kernel still runs (L2 is
+        // coherent: what that kernel writes is what the loads below return)
+        const int64_t r = static_cast<int64_t>(blockIdx.x) * kRows + threadIdx.x / TPR;
+        if (r < rows) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+                if (c < cols)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(x + r * ldx + c));
+            }
+        }
+    }
+    grid_dependency_wait();
     int flip = 0;
     for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRows; r0 < rows;
          r0 += static_cast<int64_t>(gridDim.x) * kRows, flip ^= 1) {
@@ -767,10 +781,10 @@ struct RowLaunch {
         const int grid = row_grid(rows, row_block<TPR>() / TPR);
         if (xa == 8)
             launch_dependent(quant_row_kernel<FMT, TPR, U, 8>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q, ldq,
-                             d, 1, qa, err);
+                             d, 1, qa, rows <= 2 * sm_count(), err);
         else
             launch_dependent(quant_row_kernel<FMT, TPR, 2 * U, 4>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q,
-                             ldq, d, xa == 4, qa, err);
+                             ldq, d, xa == 4, qa, rows <= 2 * sm_count(), err);
     }
 };
 
