@@ -456,8 +456,9 @@ typedef struct {
 int gemm_fp8_dense_plan(int64_t M, int64_t N, int64_t K, int out_dtype, fp8_gemm_plan_info *info);
 
 /* How gemm_fp8_mx would run a block-scaled problem now: mt 3 (CTA pairs,
- * 256 x 256 tiles, one accumulator per CTA, scale chunks loaded by TMA) or
- * mt 1 with bn 256 or 128 (128-row tiles).  FP8_ERR_SHAPE unless K % 32 == 0. */
+ * 256 x 256 tiles, scale chunks loaded by TMA) or mt 1 with bn 256 or 128, or
+ * 64, 32 or 16 for products that narrow (128-row tiles, skinny ones split
+ * along K).  FP8_ERR_SHAPE unless K % 32 == 0. */
 int gemm_fp8_mx_plan(int64_t M, int64_t N, int64_t K, int out_dtype, fp8_gemm_plan_info *info);
 
 /* How gemm_fp8_sparse24 would run an M x N x K 2:4 problem now: mt 3 (CTA

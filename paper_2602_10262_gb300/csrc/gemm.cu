@@ -85,12 +85,12 @@ constexpr int SPARSE_BN_MAX_MT2 = 224;
 // (2 KB each), then the B chunks: 4 / 5 / 7 / 8 stages for BNC = 128 / 64 /
 // 32 / 16, each k-block's metadata in its own 4 TMEM columns.  Launches
 // mixing dense and sparse problems, BNC = 256 and MT = 2 keep KC = 1.
-// MX: block-scaled launches (kind::mxf8f6f4): 128 x 128 or 128 x 256 tiles
-// or CTA pairs, dense codes as above, and per k-block 512-byte chunks of
+// MX: block-scaled launches (kind::mxf8f6f4): 128 x 16 .. 128 x 128 or 128 x
+// 256 tiles or CTA pairs, dense codes as above, and per k-block 512-byte chunks of
 // E8M0 scales after the B chunks (A's 128 rows, then B's, 128 rows per
 // chunk; a pair's CTA holds all 256 rows of B's), copied into a ring of
-// TMEM columns (per k-block A's 4, then 4 per 128 rows of B): columns
-// 128..255 beside the first of two accumulators for 128-wide tiles, from
+// TMEM columns (per k-block A's 4, then 4 per 128 rows of B): beside the
+// first of two accumulators for tiles up to 128 wide, from
 // column 256 after the single accumulator for 256-wide ones and pairs
 // (MX = 1).  One accumulator stops the tensor pipe for every tile's
 // epilogue, so pairs with more than one tile each (MX = 2) keep a ring of
@@ -136,7 +136,7 @@ struct Cfg {
     static constexpr int kSfChunk = 512;                        // scales of 128 rows x one k-block
     // MX: 128-row scale chunks of B per k-block (a pair's MMA reads all 256
     // rows' scales from each CTA's tensor memory, so each CTA holds both)
-    static constexpr int kSfQ = MX ? BNC / 128 : 0;
+    static constexpr int kSfQ = MX ? (BNC > 128 ? BNC / 128 : 1) : 0;
     // MX: A's chunk and B's chunks of each k-block, rounded up to whole
     // swizzle atoms
     static constexpr int kSfBytes = MX ? (KC * (1 + kSfQ) * kSfChunk + 1023) / 1024 * 1024 : 0;
@@ -180,8 +180,8 @@ struct Cfg {
     static_assert(!PAIR || (MT == 1 && KC == 2 && BNC == (SP ? SPARSE_BN_MAX_MT2 : BN_MAX)),
                   "CTA pairs: dense 256 x 256 or 2:4 256 x 224 tiles");
     static_assert(kBChunk % 1024 == 0, "B chunks stay swizzle-atom aligned");
-    static_assert(!MX || (MT == 1 && !SP && (BNC == 128 || (BNC == BN_MAX && (KC == 1 || PAIR)))),
-                  "block-scaled launches: 128-row dense tiles, 128 or 256 wide, or CTA pairs");
+    static_assert(!MX || (MT == 1 && !SP && (BNC <= 128 || (BNC == BN_MAX && (KC == 1 || PAIR)))),
+                  "block-scaled launches: 128-row dense tiles, up to 128 or 256 wide, or CTA pairs");
     static_assert(!MX || kSfCol0 + kSfCols * kSfSlots <= (kOverlap || kAcc == 1 ? TMEM_COLS : BN_MAX),
                   "scale ring fits beside the accumulators");
     static_assert(!kOverlap || (kAcc1 >= BN_MAX - kDrainFirst && kAcc1 < BN_MAX),
@@ -447,7 +447,8 @@ __device__ __forceinline__ void tmem_sums16(uint32_t taddr, float (&v)[16])
 // Split-K within a cluster (one unit per CTA, the slices of a tile as the
 // CTAs of one cluster, rank = slice).  Slice r > 0 writes its partial sums
 // into the rank-0 CTA's shared memory, column by column (element (row, col)
-// of slice r at ((r - 1) * bn + col) * rows_per_tile + row floats from `to`).
+// of slice r at ((r - 1) * cols + col) * rows_per_tile + row floats from
+// `to`; cols: the tile's columns of C, rounded up to 16).
 // Where they fit beside the TMA ring (in the staging buffers, which a split
 // tile's epilogue does not use) they are sent at once; else into the ring,
 // once the rank-0 CTA has said that its MMAs are done with it.  That
@@ -455,11 +456,12 @@ __device__ __forceinline__ void tmem_sums16(uint32_t taddr, float (&v)[16])
 // sum took longer than the k-loop of 16 x 4096 x 4096 (3.6 against 1.5 us):
 // with its quantise that launch takes 9.2 us, 10.4 before, 64 x 8192 x 8192
 // 17.1 (19.1), 2:4 64 x 8192 x 8192 14.0 (16.0).
-__device__ __forceinline__ void cluster_send_partial(const ProblemScalars& P, uint32_t to, int rows_per_tile,
-                                                     int slice, int row, uint32_t taddr, int c_lo, int c_hi)
+__device__ __forceinline__ void cluster_send_partial(uint32_t to, int rows_per_tile,
+                                                     int cols, int slice, int row, uint32_t taddr, int c_lo,
+                                                     int c_hi)
 {
-    const uint32_t base = to + 4u * static_cast<uint32_t>((slice - 1) * P.bn * rows_per_tile + row);
-    for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+    const uint32_t base = to + 4u * static_cast<uint32_t>((slice - 1) * cols * rows_per_tile + row);
+    for (int c0 = c_lo; c0 < min(c_hi, cols); c0 += 16) {
         float v[16];
         tmem_sums16(taddr + c0, v);
 #pragma unroll
@@ -472,14 +474,16 @@ __device__ __forceinline__ void cluster_send_partial(const ProblemScalars& P, ui
 // then the other slices' from `recv` (this row's first float), added in slice
 // order (the same sums as the global split path).
 __device__ __forceinline__ void cluster_sums16(const ProblemScalars& P, const float* recv, int rows_per_tile,
-                                               uint32_t taddr, int c, float (&acc)[16])
+                                               int cols, uint32_t taddr, int c, float (&acc)[16])
 {
     tmem_sums16(taddr + c, acc);
 #pragma unroll
     for (int t = 0; t < 16; ++t)
         acc[t] = __fadd_rn(0.0f, acc[t]);
+    if (c >= cols)                                    // past C: nothing was sent
+        return;
     for (int sl = 1; sl < P.splits; ++sl) {
-        const float* col = recv + ((sl - 1) * P.bn + c) * rows_per_tile;
+        const float* col = recv + ((sl - 1) * cols + c) * rows_per_tile;
 #pragma unroll
         for (int t = 0; t < 16; ++t)
             acc[t] = __fadd_rn(acc[t], col[t * rows_per_tile]);
@@ -790,7 +794,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     // them on the critical path).
     const int total_tiles = prm.total_tiles;
     // (only one-problem launches add slices up within clusters)
-    constexpr bool kCanSplitCluster = MAXP == 1 && !PAIR && MX == 0;
+    constexpr bool kCanSplitCluster = MAXP == 1 && !PAIR && (MX == 0 || BNC <= 128);
     const int cluster_split = kCanSplitCluster ? prm.cluster_split : 0;
     int* const err = prm.err;
     const unsigned long long wlim = prm.wait_ns;
@@ -1371,7 +1375,8 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                     break;
                 }
                 const int rows_per_tile = BM * MT;
-                const bool beside = (P.splits - 1) * P.bn * rows_per_tile * 4 <= C::kEpiBytes;
+                const int cols = min(P.bn, (P.rows_q - jbase + 15) & ~15);
+                const bool beside = (P.splits - 1) * cols * rows_per_tile * 4 <= C::kEpiBytes;
                 uint8_t* recv = beside ? epi_smem : smem;
                 if (!cluster_waited)
                     cluster_wait();                     // every CTA of the cluster is up
@@ -1388,7 +1393,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                     }
                     const float* mine = reinterpret_cast<const float*>(recv) + row;
                     const auto load = [&](int c, float (&v)[16]) {
-                        cluster_sums16(P, mine, rows_per_tile, taddr, c, v);
+                        cluster_sums16(P, mine, rows_per_tile, cols, taddr, c, v);
                     };
                     // staging buffers: whichever of the two regions the
                     // partial sums are not in
@@ -1419,7 +1424,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                         abort_pipeline(abort_flag, err);
                         break;
                     }
-                    cluster_send_partial(P, cluster_map(smem_u32(recv), 0u), rows_per_tile, crank, row, taddr, c_lo,
+                    cluster_send_partial(cluster_map(smem_u32(recv), 0u), rows_per_tile, cols, crank, row, taddr, c_lo,
                                          c_hi);
                     mbar_arrive_remote(cluster_map(split_written_bar, 0u));
                 }
@@ -1798,9 +1803,16 @@ int slice_kblocks(int k_blocks, int s)
 int split_count(const Job& j)
 {
     const int sms = sm_count();
-    if (j.sfp != nullptr || !splits_k(j.rows_p, j.rows_q, j.K))
+    if (j.rows_p <= 0 || j.rows_q <= 0)
         return 1;
-    const int64_t tiles = problem_tiles(j.rows_p, j.rows_q, j.K);
+    // block-scaled products run 128 x 128 tiles there: one column of them.
+    // 128 x 8192 x 8192 took 28.6 us unsplit, 21.4 in two slices; 16 x 4096 x
+    // 14336 40.5 and 16.4 in four.
+    const int64_t mx_tiles = (j.rows_p + BM - 1) / BM;
+    if (j.sfp ? (j.K + BK - 1) / BK < 32 || j.rows_q > 128 || 2 * mx_tiles > sms
+              : !splits_k(j.rows_p, j.rows_q, j.K))
+        return 1;
+    const int64_t tiles = j.sfp ? mx_tiles : problem_tiles(j.rows_p, j.rows_q, j.K);
     const int k_blocks = static_cast<int>((j.K + BK - 1) / BK);
     int s = std::min<int64_t>(8, sms / tiles);
     s = std::min(s, k_blocks / 8);
@@ -2295,8 +2307,11 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
                            : plan<MAXP, 1, false, BN_MAX, 2, 1, true>(prm, max_ctas, pl);
             if (max_bn > 128)
                 return plan<MAXP, 1, false, BN_MAX, 1, 1>(prm, max_ctas, pl);
-            return kc == 2 ? plan<MAXP, 1, false, 128, 2, 1>(prm, max_ctas, pl)
-                           : plan<MAXP, 1, false, 128, 1, 1>(prm, max_ctas, pl);
+            if (max_bn <= 16)
+                return plan<MAXP, 1, false, 16, 2, 1>(prm, max_ctas, pl);
+            if (max_bn <= 64)
+                return plan<MAXP, 1, false, 64, 2, 1>(prm, max_ctas, pl);
+            return plan<MAXP, 1, false, 128, 2, 1>(prm, max_ctas, pl);
         }
         return FP8_ERR_UNSUPPORTED;
     }
@@ -2639,9 +2654,15 @@ int run_jobs(Params<MAXP>& prm, const Job* jobs, const int* bns, int n, int max_
 
 // N width of a block-scaled launch: 256 (CTA pairs, or 128 x 256 tiles with
 // two 128-row scale chunks of B per k-block) where the problem has enough
-// tiles for it, else 128.
+// tiles for it; 16, 32 or 64 where that covers a skinny product's Q side (one
+// column of tiles, whose scales are one 128-row chunk; a 128-row box of B is
+// written to shared memory whatever C needs of it); else 128.  16 x 14336 x
+// 4096: 13.5 us 16 wide, 22.1 us 128 wide; 16 x 4096 x 4096 (split) 8.4 and
+// 14.5.
 int mx_tile_width(const Job& j)
 {
+    if (j.rows_q <= 64)
+        return j.rows_q <= 16 ? 16 : (j.rows_q <= 32 ? 32 : 64);
     return pick_bn(j.rows_p, j.rows_q, j.K, BN_MAX) == BN_MAX ? BN_MAX : 128;
 }
 
@@ -2801,7 +2822,7 @@ extern "C" int gemm_fp8_mx_plan(int64_t M, int64_t N, int64_t K, int out_dtype, 
                      N, out_dtype, 0, FP8_E4M3, FP8_E4M3);
     j.sfp = fake;
     j.sfq = fake;
-    return describe_plan(j, mx_tile_width(j), false, M, N, info);
+    return describe_plan(j, mx_tile_width(j), true, M, N, info);
 }
 
 // ---------------------------------------------------------------- no-allocation variant
@@ -2925,7 +2946,7 @@ extern "C" int gemm_fp8_mx(int64_t M, int64_t N, int64_t K, const uint8_t* A, in
     const int bn = mx_tile_width(j);
     Params<1> prm;
     memset(&prm, 0, sizeof(prm));
-    return run_jobs(prm, &j, &bn, 1, 0, st);
+    return run_jobs(prm, &j, &bn, 1, 0, st, nullptr, true);
 }
 
 extern "C" int gemm_fp8_sparse24(int64_t M, int64_t N, int64_t K, const uint8_t* a_vals,

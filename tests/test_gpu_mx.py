@@ -348,6 +348,22 @@ def test_mx_pairs_stalled_launch_times_out(gb):
 @pytest.mark.parametrize("M,N,K,out", [(2560, 2560, 4096, 0), (5120, 2816, 128, 0), (5200, 2800, 416, 1),
                                        (5120, 5001, 672, 0), (7680, 7680, 160, 1)])
 def test_mx_pair_tile_counts_exact(gb, M, N, K, out):
+    assert gb.gemm_fp8_mx_plan(M, N, K, out)["mt"] == 3
+    _check_mx_exact(gb, M, N, K, out)
+
+
+# skinny products split along K within clusters: partial sums beside the ring
+# and in it, two to eight slices, ragged everything
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(1, 520, 4096), (16, 8192, 4096), (17, 1029, 4128), (33, 4096, 8192),
+                                   (64, 1544, 8224), (100, 777, 8192), (128, 8192, 8192), (128, 256, 16384)])
+def test_mx_split_clusters_exact(gb, M, N, K, out):
+    plan = gb.gemm_fp8_mx_plan(M, N, K, out)
+    assert plan["mt"] == 1 and plan["splits"] > 1, plan
+    _check_mx_exact(gb, M, N, K, out)
+
+
+def _check_mx_exact(gb, M, N, K, out):
     """Integers times powers of two: every partial sum is exact in FP32, so
     the product equals float64's."""
     A = _dev(workloads.small_int_codes((M, K), seed=M))
@@ -363,7 +379,6 @@ def test_mx_pair_tile_counts_exact(gb, M, N, K, out):
         return (v * torch.exp2(s.double() - 127)[:, :, None]).reshape(codes.shape)
 
     (sa, ta), (sb, tb) = scales(M), scales(N)
-    assert gb.gemm_fp8_mx_plan(M, N, K, out)["mt"] == 3
     C = gb.gemm_fp8_mx(A, ta, B, tb, out_dtype=out)
     assert gb.fp8_last_device_error() == 0
     ref = value(A, sa) @ value(B, sb).T
