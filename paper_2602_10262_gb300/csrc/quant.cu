@@ -891,117 +891,87 @@ __device__ __forceinline__ int64_t mx_tiled_offset(int64_t r, int64_t b, int64_t
     return 512 * ((r >> 7) * kb + (b >> 2)) + 16 * (r & 31) + 4 * ((r & 127) >> 5) + (b & 3);
 }
 
-// One warp quantises a 128-column window of one row at a time: lane l
-// holds columns 4l .. 4l + 3, so the 32-element block j (of four) is lanes
-// 8j .. 8j + 7, and its amax is an 8-lane max reduction.  For a non-zero
-// block, e = floor(log2 amax) - emax (emax 8 for E4M3, 15 for E5M2) read
-// from amax's exponent field (a subnormal amax gives the floor -127), so
-// amax * 2^-e lies in [2^emax, 2^(emax+1)); the scale code is e + 127 and the
-// codes are the format's round-to-nearest-even, saturating encoding of the
-// IEEE product x * 2^-e (exact unless it falls below 2^-126).  An all-zero
-// block gets scale code 0 and the codes of its (signed) zeros.
-// Grid: blockIdx.y walks rows (with a stride past 65535), blockIdx.x takes
-// mx_windows<TILED>() consecutive windows of the row: warp w of the block
-// handles windows x * that + w + 8 u (u < mx_unroll<TILED>()), all loads
-// issued before any arithmetic.  Measured: eight loads in flight per lane
-// suit the tiled scale layout, four the row-major one (eight made it 25 %
-// slower).
-template <int TILED>
-__host__ __device__ constexpr int mx_unroll()
-{
-    return TILED ? 8 : 4;
-}
-
-template <int TILED>
-__host__ __device__ constexpr int mx_windows()
-{
-    return (kThreads / 32) * mx_unroll<TILED>();   // windows per block and row
-}
-
+// One warp quantises a 256-column window of one row at a time: lane l holds
+// columns 8l .. 8l + 7, so a 32-element block is four lanes, and its amax is
+// their local maxima and two shuffles.  For a non-zero block, e = floor(log2
+// amax) - emax (emax 8 for E4M3, 15 for E5M2) read from amax's exponent field
+// (a subnormal amax gives the floor -127), so amax * 2^-e lies in [2^emax,
+// 2^(emax+1)); the scale code is e + 127 and the codes are the format's
+// round-to-nearest-even, saturating encoding of the IEEE product x * 2^-e
+// (exact unless it falls below 2^-126).  An all-zero block gets scale code 0
+// and the codes of its (signed) zeros.  The four codes of a 128-column
+// k-block are joined over its 16 lanes and leave as one word.
+// The windows of the matrix are one list, the row by one 32-bit division, a
+// warp takes one at a time; with the tiled scale layout the list goes on over
+// the padding rows of the last 128, whose scales are 1 (a memset before it
+// kept the launch from overlapping the kernel before).  What bounds it beside
+// HBM is instructions: 128-column windows of four columns a lane spent twice
+// as many on the same data (4096 x 4096 19.5 us, 15.0 now; 4096 x 14336 54.8,
+// 46.5; 16384 x 8192 112, 103; 16 x 4096 3.6, 2.0).  Two, four or eight
+// windows a warp at once, loads first, were slower (16.7, 17.6 and 23.9 us at
+// 4096 x 4096): enough warps have a load in flight.
 template <int FMT, int TILED>
 __global__ void __launch_bounds__(kThreads) quant_mx_kernel(const float* __restrict__ x, int64_t rows,
-                                                            int64_t cols, int64_t ldx, uint8_t* __restrict__ q,
-                                                            int64_t ldq, uint8_t* __restrict__ sc, int vec,
-                                                            int qvec, int* err)
+                                                            int64_t cols, int64_t ldx, int xa,
+                                                            uint8_t* __restrict__ q, int64_t ldq, int qa,
+                                                            uint8_t* __restrict__ sc, int* err)
 {
     grid_launch_dependents();
     grid_dependency_wait();
     constexpr int kEmax = FMT == 1 ? 15 : 8;
-    constexpr int kMxU = mx_unroll<TILED>();
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
     const int64_t kb = (cols + 127) / 128;
-    const int64_t win0 = static_cast<int64_t>(blockIdx.x) * mx_windows<TILED>() + warp;
-    for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        const float* xr = x + r * ldx;
-        float4 v[kMxU];
-        bool in[kMxU];
-#pragma unroll
-        for (int u = 0; u < kMxU; ++u) {
-            const int64_t c0 = (win0 + u * (kThreads / 32)) * 128 + 4 * lane;
-            in[u] = c0 < cols;                                // cols % 32 == 0: whole blocks in or out
-            v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (in[u]) {
-                if (vec)
-                    v[u] = __ldg(reinterpret_cast<const float4*>(xr + c0));
-                else
-                    v[u] = make_float4(xr[c0], xr[c0 + 1], xr[c0 + 2], xr[c0 + 3]);
-            }
+    const int64_t segs = (cols + 255) / 256;
+    const int64_t total = (TILED ? (rows + 127) / 128 * 128 : rows) * segs;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads / 32);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); i < total; i += step) {
+        int64_t r, seg;
+        if (total <= 0xFFFFFFFFll) {
+            const uint32_t n = static_cast<uint32_t>(segs), g = static_cast<uint32_t>(i) / n;
+            r = g;
+            seg = static_cast<uint32_t>(i) - g * n;
+        } else {
+            r = i / segs;
+            seg = i - r * segs;
         }
+        const int64_t c = seg * 256 + 8 * lane;
+        const bool in = c < cols && r < rows;     // cols % 32 == 0: a lane's eight columns are all in or out
+        float v[8];
+        load_8(x + r * ldx + c, in ? 8 : 0, xa, v);
+        uint32_t m = 0;
 #pragma unroll
-        for (int u = 0; u < kMxU; ++u) {
-            const int64_t w = win0 + u * (kThreads / 32);
-            if (w >= kb)
-                break;                                        // the whole warp leaves together
-            const int64_t c0 = w * 128 + 4 * lane;
-            uint32_t m = max(max(abs_bits(v[u].x), abs_bits(v[u].y)), max(abs_bits(v[u].z), abs_bits(v[u].w)));
-            m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-            m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-            m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 4));
-            if (m >= kInfBits && (lane & 7) == 0)
-                report_device_error(err, FP8_ERR_NONFINITE);
-            uint32_t code = 0;
-            float s = 1.0f;
-            if (m != 0u && m < kInfBits) {
-                const int E = static_cast<int>(m >> 23);  // biased exponent of amax
-                const int e = E == 0 ? -127 : max(E - 127 - kEmax, -127);
-                code = static_cast<uint32_t>(e + 127);
-                s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);     // 2^-e, normal
-            }
-            if (in[u]) {
-                const uint32_t word = enc4<FMT>(v[u], s);
-                uint8_t* qd = q + r * ldq + c0;
-                if (qvec) {
-                    *reinterpret_cast<uint32_t*>(qd) = word;
-                } else {
-                    qd[0] = word & 0xFFu;
-                    qd[1] = (word >> 8) & 0xFFu;
-                    qd[2] = (word >> 16) & 0xFFu;
-                    qd[3] = word >> 24;
-                }
-            }
-            // the four blocks' scale codes, from lanes 0, 8, 16, 24
-            const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, code, 0), s1 = __shfl_sync(0xFFFFFFFFu, code, 8);
-            const uint32_t s2 = __shfl_sync(0xFFFFFFFFu, code, 16), s3 = __shfl_sync(0xFFFFFFFFu, code, 24);
-            if (lane == 0) {
-                const int64_t b0 = w * 4;                         // first block of the window
-                const int nb = static_cast<int>(min(static_cast<int64_t>(4), cols / 32 - b0));
-                const uint32_t sj[4] = {s0, s1, s2, s3};
-                if (TILED) {
-                    uint32_t word = 0;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        word |= (j < nb ? sj[j] : 127u) << (8 * j);     // blocks past cols: scale 1
-                    *reinterpret_cast<uint32_t*>(sc + mx_tiled_offset(r, b0, kb)) = word;
-                } else {
-                    uint8_t* sr = sc + r * (cols / 32) + b0;
-                    if (nb == 4 && (reinterpret_cast<uintptr_t>(sr) & 3u) == 0) {
-                        *reinterpret_cast<uint32_t*>(sr) = s0 | (s1 << 8) | (s2 << 16) | (s3 << 24);
-                    } else {
-                        for (int j = 0; j < nb; ++j)
-                            sr[j] = static_cast<uint8_t>(sj[j]);
-                    }
-                }
+        for (int k = 0; k < 8; ++k)
+            m = max(m, abs_bits(v[k]));
+        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+        if (m >= kInfBits && (lane & 3) == 0)
+            report_device_error(err, FP8_ERR_NONFINITE);
+        uint32_t code = 0;
+        float s = 1.0f;
+        if (m != 0u && m < kInfBits) {
+            const int E = static_cast<int>(m >> 23);  // biased exponent of amax
+            const int e = E == 0 ? -127 : max(E - 127 - kEmax, -127);
+            code = static_cast<uint32_t>(e + 127);
+            s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);     // 2^-e, normal
+        }
+        store_codes<FMT, 8>(q + r * ldq + c, in ? 8 : 0, qa, v, s);
+        // blocks past cols and padding rows: scale 1
+        uint32_t word = (in ? code : 127u) << (8 * ((lane >> 2) & 3));
+        word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
+        word |= __shfl_xor_sync(0xFFFFFFFFu, word, 8);
+        const int64_t k = 2 * seg + (lane >> 4);              // k-block of this half warp
+        if ((lane & 15) != 0 || k >= kb)
+            continue;
+        if (TILED) {
+            *reinterpret_cast<uint32_t*>(sc + mx_tiled_offset(r, 4 * k, kb)) = word;
+        } else {
+            uint8_t* sr = sc + r * (cols / 32) + 4 * k;
+            const int nb = static_cast<int>(min(static_cast<int64_t>(4), cols / 32 - 4 * k));
+            if (nb == 4 && (reinterpret_cast<uintptr_t>(sr) & 3u) == 0) {
+                *reinterpret_cast<uint32_t*>(sr) = word;
+            } else {
+                for (int j = 0; j < nb; ++j)
+                    sr[j] = static_cast<uint8_t>(word >> (8 * j));
             }
         }
     }
@@ -1056,29 +1026,17 @@ int quantize_mx(const float* x, int64_t rows, int64_t cols, int64_t ldx, uint8_t
         return FP8_ERR_ALIGN;
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
-    const int vec = aligned16(x) && (ldx % 4 == 0);
-    const int qvec = (reinterpret_cast<uintptr_t>(q) % 4 == 0) && (ldq % 4 == 0);
-    // a few blocks per SM, each walking rows (short-lived blocks cost more
+    const int xa = row_align(x, ldx, 4), qa = row_align(q, ldq, 1);
+    // a few blocks per SM, each walking windows (short-lived blocks cost more
     // in launch and tail than they save)
-    const int64_t kb = (cols + 127) / 128;
-    const int64_t win = layout == 1 ? mx_windows<1>() : mx_windows<0>();
-    const int64_t gx = (kb + win - 1) / win;
-    int64_t gy = std::min<int64_t>(rows, static_cast<int64_t>(sm_count()) * 16 / gx);
-    gy = std::max<int64_t>(1, std::min<int64_t>(gy, 65535));
-    const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy));
-    if (layout == 1) {
-        int* err = device_error_word();
-        if (rows % 128 != 0) {                   // padding rows of the last tile: scale 1
-            GB_CUDA_OK(cudaMemsetAsync(scales, 127, fp8_mx_scale_tiled_bytes(rows, cols), st));
-            quant_mx_kernel<FMT, 1><<<grid, kThreads, 0, st>>>(x, rows, cols, ldx, q, ldq, scales, vec, qvec, err);
-        } else {
-            launch_dependent(quant_mx_kernel<FMT, 1>, grid, kThreads, st, x, rows, cols, ldx, q, ldq, scales, vec,
-                             qvec, err);
-        }
-    } else {
-        launch_dependent(quant_mx_kernel<FMT, 0>, grid, kThreads, st, x, rows, cols, ldx, q, ldq, scales, vec, qvec,
-                         device_error_word());
-    }
+    const int64_t windows = (layout == 1 ? (rows + 127) / 128 * 128 : rows) * ((cols + 255) / 256);
+    const int64_t per_block = kThreads / 32;
+    const int grid = static_cast<int>(std::min<int64_t>((windows + per_block - 1) / per_block, sm_count() * 16));
+    int* err = device_error_word();
+    if (layout == 1)
+        launch_dependent(quant_mx_kernel<FMT, 1>, grid, kThreads, st, x, rows, cols, ldx, xa, q, ldq, qa, scales, err);
+    else
+        launch_dependent(quant_mx_kernel<FMT, 0>, grid, kThreads, st, x, rows, cols, ldx, xa, q, ldq, qa, scales, err);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }

@@ -386,3 +386,24 @@ def _check_mx_exact(gb, M, N, K, out):
         assert torch.equal(C.double(), ref)
     else:
         assert torch.equal(C, ref.float().bfloat16())
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(1, 32), (3, 224), (129, 256), (5, 288), (128, 384), (300, 4128)])
+def test_mx_quantize_alignments(gb, orc, layout, rows, cols):
+    """256-column windows that end in a row, padding rows, and every row
+    alignment of x and q; bytes between q's rows untouched."""
+    x = _mx_inputs(rows, cols, seed=rows + cols)
+    q_ref, s_ref = orc.mx_quantize(x, 0)
+    want = s_ref if layout == 0 else tiled_layout(s_ref, rows, cols)
+    for pad, off, qpad, qoff in ((0, 0, 0, 0), (4, 4, 4, 4), (1, 1, 1, 1)):
+        xb = torch.full((rows * (cols + pad) + off,), float("nan"), device="cuda")
+        xt = xb[off:].view(rows, cols + pad)[:, :cols]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((rows * (cols + qpad) + qoff,), 0xA5, dtype=torch.uint8, device="cuda")
+        qt = qb[qoff:].view(rows, cols + qpad)[:, :cols]
+        _, s = gb.fp8_quantize_mx(xt, 0, scale_layout=layout, q=qt)
+        assert np.array_equal(qt.cpu().numpy(), q_ref)
+        assert np.array_equal(s.cpu().numpy(), want)
+        assert bool((qb[qoff:].view(rows, cols + qpad)[:, cols:] == 0xA5).all())
+    assert gb.fp8_last_device_error() == 0
