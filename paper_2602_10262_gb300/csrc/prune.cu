@@ -6,7 +6,10 @@
 // store of the four metadata nibbles.  Rows whose length or alignment does
 // not allow it take the same pieces with narrower accesses.
 // Bandwidth-bound: 1 byte read, 0.625 bytes written per element; no
-// allocation, one launch.  The inverse moves the same bytes the other way.
+// allocation, one launch.  Loads are ordinary ones (of whole pieces, at L2):
+// these kernels may start before their input is written (launch_dependent),
+// which the read-only path does not allow.  The inverse moves the same bytes
+// the other way.
 #include <algorithm>
 
 #include "common.cuh"
@@ -55,7 +58,7 @@ __global__ void __launch_bounds__(kThreads) prune24_vec_kernel(const uint8_t* __
         for (int u = 0; u < U; ++u) {
             const int p = p_first + u * kThreads;
             if (p < pieces)
-                x[u] = __ldg(src + p);
+                x[u] = __ldcg(src + p);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -105,31 +108,31 @@ __device__ __forceinline__ void load_words(const uint8_t* p, int n, int align, u
     for (int i = 0; i < W; ++i)
         w[i] = 0;
     if (W == 4 && align >= 16 && n == 16) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+        const uint4 v = __ldca(reinterpret_cast<const uint4*>(p));
         w[0] = v.x, w[W > 1 ? 1 : 0] = v.y, w[W > 2 ? 2 : 0] = v.z, w[W > 3 ? 3 : 0] = v.w;
     } else if (W >= 2 && align >= 8 && n == 4 * W) {
 #pragma unroll
         for (int i = 0; i + 1 < W; i += 2) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + 4 * i));
+            const uint2 v = __ldca(reinterpret_cast<const uint2*>(p + 4 * i));
             w[i] = v.x, w[i + 1] = v.y;
         }
     } else if (align >= 4) {
 #pragma unroll
         for (int i = 0; i < W; ++i)
             if (4 * i + 4 <= n)
-                w[i] = __ldg(reinterpret_cast<const uint32_t*>(p + 4 * i));
+                w[i] = __ldca(reinterpret_cast<const uint32_t*>(p + 4 * i));
             else if (4 * i + 2 <= n)
-                w[i] = __ldg(reinterpret_cast<const uint16_t*>(p + 4 * i));
+                w[i] = __ldca(reinterpret_cast<const uint16_t*>(p + 4 * i));
     } else if (align >= 2) {
 #pragma unroll
         for (int i = 0; i < 2 * W; ++i)
             if (2 * i + 2 <= n)
-                w[i / 2] |= static_cast<uint32_t>(__ldg(reinterpret_cast<const uint16_t*>(p + 2 * i))) << (16 * (i & 1));
+                w[i / 2] |= static_cast<uint32_t>(__ldca(reinterpret_cast<const uint16_t*>(p + 2 * i))) << (16 * (i & 1));
     } else {
 #pragma unroll
         for (int i = 0; i < 4 * W; ++i)
             if (i < n)
-                w[i / 4] |= static_cast<uint32_t>(__ldg(p + i)) << (8 * (i & 3));
+                w[i / 4] |= static_cast<uint32_t>(__ldca(p + i)) << (8 * (i & 3));
     }
 }
 
@@ -232,8 +235,8 @@ __global__ void __launch_bounds__(kThreads) decompress24_vec_kernel(const uint2*
         for (int u = 0; u < U; ++u) {
             const int64_t p = p0 + u * kThreads;
             if (p < pieces) {
-                v[u] = __ldg(vals + p);
-                n[u] = __ldg(meta + p);
+                v[u] = __ldcg(vals + p);
+                n[u] = __ldcg(meta + p);
             }
         }
 #pragma unroll
@@ -270,11 +273,11 @@ __global__ void __launch_bounds__(kThreads) decompress24_any_kernel(const uint8_
                 load_words<2>(vals + r[u] * s.ldv + 8 * p[u], 2 * n[u], v_align, v[u]);
                 const uint8_t* md = meta + r[u] * s.ldm + 2 * p[u];
                 if (m_align >= 2 && n[u] > 2) {
-                    m[u] = __ldg(reinterpret_cast<const uint16_t*>(md));
+                    m[u] = __ldca(reinterpret_cast<const uint16_t*>(md));
                 } else {
-                    m[u] = __ldg(md);
+                    m[u] = __ldca(md);
                     if (n[u] > 2)
-                        m[u] |= static_cast<uint32_t>(__ldg(md + 1)) << 8;
+                        m[u] |= static_cast<uint32_t>(__ldca(md + 1)) << 8;
                 }
             }
         }

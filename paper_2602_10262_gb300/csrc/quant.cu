@@ -18,6 +18,12 @@
 // backwards, its end being what is left in L2), and a one-thread kernel turns
 // the slot into d = amax / 448.
 //
+// Most of these kernels start before the one that writes their input has
+// ended (programmatic serialization): their loads are ordinary or L2 ones,
+// never the read-only path, whose data may not change while a kernel runs.
+// The kernels that read long rows twice are launched plainly and do use it
+// (1024 x 32768: 48 us, 57 with ordinary loads; held in registers 30).
+//
 // The scale is s = T / amax with an IEEE-rounded division (__fdiv_rn), T the
 // format's largest finite value (448 for E4M3, 57344 for E5M2), and each code
 // is cvt.rn.satfinite of the IEEE product x * s (__fmul_rn) to that format.
@@ -119,9 +125,10 @@ __device__ __forceinline__ void scale_from_amax(uint32_t amax_bits, float& s, fl
 // TB/s), 16384 x 14336 183 -> 165 us (7.1 TB/s), 16384 x 512 28.5 -> 8.5 us,
 // 16 x 14336 3.4 -> 2.5 us.  Fused with 2:4 compression: 14336 x 4096 64.7
 // -> 50.2 us (6.6 TB/s), 16384 x 16384 250 -> 216 us (its ALU pipe was 68 %
-// busy: the four-group selection took half of that away).
+// busy: the four-group selection took half of that away).  1024 x 32768 47.7
+// -> 29.8 us.
 constexpr int kRowBlock = 256;            // threads of a block where TPR is smaller
-constexpr int kRowMaxCols = 16384;        // longest row held in registers
+constexpr int kRowMaxCols = 32768;        // longest row held in registers
 
 template <int TPR>
 constexpr int row_block()
@@ -141,13 +148,13 @@ __device__ __forceinline__ void load_vec(const float* p, int64_t left, bool vec,
                            "=f"(v[7])
                          : "l"(p));
         } else {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+            const float4 a = __ldca(reinterpret_cast<const float4*>(p));
             v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
         }
     } else {
 #pragma unroll
         for (int i = 0; i < W; ++i)
-            v[i] = i < left ? __ldg(p + i) : 0.0f;
+            v[i] = i < left ? __ldca(p + i) : 0.0f;
     }
 }
 
@@ -155,8 +162,8 @@ __device__ __forceinline__ void load_vec(const float* p, int64_t left, bool vec,
 __device__ __forceinline__ void load_two_vec4(const float* p, int64_t left, float (&v)[8])
 {
     const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    const float4 a = left > 0 ? __ldg(reinterpret_cast<const float4*>(p)) : z;
-    const float4 b = left > 0 ? __ldg(reinterpret_cast<const float4*>(p) + 1) : z;
+    const float4 a = left > 0 ? __ldca(reinterpret_cast<const float4*>(p)) : z;
+    const float4 b = left > 0 ? __ldca(reinterpret_cast<const float4*>(p) + 1) : z;
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
     v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
 }
@@ -407,7 +414,6 @@ __global__ void __launch_bounds__(kThreads) quant_long_row_kernel(const float* _
                                                                   int vec, int* err)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     __shared__ uint32_t red[kThreads / 32];
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
         quantize_row<FMT>(x + r * ldx, cols, q + r * ldq, d + r, vec, err, red);
@@ -424,7 +430,6 @@ __global__ void __launch_bounds__(kThreads) quant_long_row_prune_kernel(const fl
                                                                         uint8_t* __restrict__ meta, int* err)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     __shared__ uint32_t red[kThreads / 32];
     const int64_t n4 = cols / 4;
     const int64_t ldv = cols / 2, ldm = cols / 8;
@@ -503,7 +508,6 @@ __global__ void __launch_bounds__(kThreads) quant_long_rows_grouped_kernel(const
                                                                            int* err)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     __shared__ uint32_t red[kThreads / 32];
     const int64_t total = jobs.row_start[jobs.n];
     for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
@@ -657,7 +661,7 @@ __global__ void __launch_bounds__(kThreads) quant_encode_kernel(const float* __r
     grid_launch_dependents();
     grid_dependency_wait();
     float s, dq;
-    scale_from_amax<FMT>(*slot, s, dq);
+    scale_from_amax<FMT>(__ldcg(slot), s, dq);
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (kThreads / 32);
     for (int64_t i0 = (static_cast<int64_t>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5)) * kItems;
          i0 < it.total; i0 += warps * kItems) {
@@ -720,8 +724,10 @@ void with_row_shape(int64_t rows, int64_t cols, F f)
             f.template operator()<128, 1>();
         else if (cols <= 4096)
             f.template operator()<512, 1>();
-        else
+        else if (cols <= 16384)
             f.template operator()<1024, 2>();
+        else
+            f.template operator()<1024, 4>();
     } else if (cols <= 256) {
         f.template operator()<32, 1>();
     } else if (cols <= 512) {
@@ -738,8 +744,10 @@ void with_row_shape(int64_t rows, int64_t cols, F f)
         f.template operator()<256, 4>();
     } else if (cols <= 12288) {
         f.template operator()<512, 3>();
-    } else {
+    } else if (cols <= 16384) {
         f.template operator()<512, 4>();
+    } else {
+        f.template operator()<1024, 4>();
     }
 }
 
@@ -830,8 +838,8 @@ int quantize(const float* x, int64_t rows, int64_t cols, int64_t ldx, int scale_
         if (cols <= kRowMaxCols)
             with_row_shape(rows, cols, RowLaunch<FMT>{x, rows, cols, ldx, q, ldq, dequant_scale, err, st});
         else
-            launch_dependent(quant_long_row_kernel<FMT>, row_grid(rows, 1), kThreads, st, x, rows, cols, ldx, q, ldq,
-                             dequant_scale, vec, err);
+            quant_long_row_kernel<FMT><<<row_grid(rows, 1), kThreads, 0, st>>>(x, rows, cols, ldx, q, ldq,
+                                                                               dequant_scale, vec, err);
         GB_CUDA_OK(cudaGetLastError());
         return FP8_OK;
     }
@@ -994,7 +1002,7 @@ __global__ void __launch_bounds__(kThreads) mx_scales_tile_kernel(const uint8_t*
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int64_t b = 4 * k + j;
-            const uint32_t v = (r < rows && b < nbr) ? src[r * nbr + b] : 127u;
+            const uint32_t v = (r < rows && b < nbr) ? __ldca(src + r * nbr + b) : 127u;
             word |= v << (8 * j);
         }
         *reinterpret_cast<uint32_t*>(dst + mx_tiled_offset(r, 4 * k, kb)) = word;
@@ -1117,8 +1125,8 @@ extern "C" int fp8_quantize_e4m3_prune24(const float* x, int64_t rows, int64_t c
     if (cols <= kRowMaxCols)
         with_row_shape(rows, cols, RowPruneLaunch{x, rows, cols, ldx, q, ldq, dequant_scale, a_vals, a_meta, err, st});
     else
-        launch_dependent(quant_long_row_prune_kernel, row_grid(rows, 1), kThreads, st, x, rows, cols, ldx, q, ldq,
-                         dequant_scale, a_vals, a_meta, err);
+        quant_long_row_prune_kernel<<<row_grid(rows, 1), kThreads, 0, st>>>(x, rows, cols, ldx, q, ldq, dequant_scale,
+                                                                            a_vals, a_meta, err);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }
@@ -1188,7 +1196,7 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
     else if (max_cols <= 32 * kGroupedTpr)
         launch(quant_rows_grouped_kernel<4, 8>, quant_rows_grouped_kernel<8, 4>);
     else
-        launch_dependent(quant_long_rows_grouped_kernel, grid, kThreads, st, rj, err);
+        quant_long_rows_grouped_kernel<<<grid, kThreads, 0, st>>>(rj, err);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }

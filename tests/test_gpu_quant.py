@@ -105,7 +105,7 @@ def test_device_encoder_all_in_range_fp32(gb, orc):
 @pytest.mark.parametrize("fmt", [0, 1])
 @pytest.mark.parametrize("rows,cols", [(r, c) for r in (9, 401) for c in
                                        (1, 31, 256, 257, 512, 513, 1024, 1025, 2048, 2049, 4096, 4097, 6144, 6145,
-                                        8192, 8199, 12288, 12289, 16384, 16385)])
+                                        8192, 8199, 12288, 12289, 16384, 16385, 32768, 32769)])
 def test_row_shapes(gb, orc, fmt, rows, cols):
     x = workloads.randn_f32((rows, cols), seed=rows + cols)
     x[rows // 2] = 0.0

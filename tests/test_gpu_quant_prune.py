@@ -99,7 +99,7 @@ def test_shape_and_alignment_rejected(gb):
 
 @pytest.mark.parametrize("rows", [5, 333])
 @pytest.mark.parametrize("cols", [128, 256, 384, 512, 640, 1024, 1152, 2048, 2176, 4096, 4224, 6144, 6272, 8192, 8320,
-                                  12288, 12416, 16384, 16512])
+                                  12288, 12416, 16384, 16512, 32768, 32896])
 def test_row_shapes(gb, rows, cols):
     """Each threads-per-row shape at its first and last column counts, with
     32- and 16-byte aligned x and 8- and 4-byte aligned outputs, equals the
