@@ -240,6 +240,7 @@ struct Params {
     float* ws;              // split-K partial sums (nullptr when no problem splits)
     unsigned* ctr;          // split-K arrival counters, zero between launches
     int cluster_split;      // > 0: one problem whose split tiles run as clusters of this many CTAs
+    int split_beside;       // cluster split-K: every tile's partial sums fit beside the TMA ring
     int mc;                 // > 0: clusters of this many CTAs take consecutive tiles of one N column;
                             // each loads 1/mc of the shared Q block and multicasts it to all
     unsigned long long wait_ns;   // limit of every bounded wait (kWaitLimitNs unless a test sets another)
@@ -449,9 +450,10 @@ __device__ __forceinline__ void tmem_sums16(uint32_t taddr, float (&v)[16])
 // into the rank-0 CTA's shared memory, column by column (element (row, col)
 // of slice r at ((r - 1) * cols + col) * rows_per_tile + row floats from
 // `to`; cols: the tile's columns of C, rounded up to 16).
-// Where they fit beside the TMA ring (in the staging buffers, which a split
-// tile's epilogue does not use) they are sent at once; else into the ring,
-// once the rank-0 CTA has said that its MMAs are done with it.  That
+// Where they fit beside the TMA ring (Params::split_beside: in the staging
+// buffers, which a split tile's epilogue does not use) they are sent at once;
+// else into the ring, once the rank-0 CTA has said that its MMAs are done with
+// it.  That
 // handshake, a cluster barrier at the end and the lane-by-lane stores of the
 // sum took longer than the k-loop of 16 x 4096 x 4096 (3.6 against 1.5 us):
 // with its quantise that launch takes 9.2 us, 10.4 before, 64 x 8192 x 8192
@@ -1376,7 +1378,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 }
                 const int rows_per_tile = BM * MT;
                 const int cols = min(P.bn, (P.rows_q - jbase + 15) & ~15);
-                const bool beside = (P.splits - 1) * cols * rows_per_tile * 4 <= C::kEpiBytes;
+                const bool beside = prm.split_beside != 0;
                 uint8_t* recv = beside ? epi_smem : smem;
                 if (!cluster_waited)
                     cluster_wait();                     // every CTA of the cluster is up
@@ -1553,13 +1555,15 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     tc_fence_before();
     __syncthreads();
     // cluster split-K: the rank-0 CTA does not leave while a peer may still
-    // write to its shared memory (nobody writes to the others', which signal
-    // and go); pairs and multicast: neither CTA frees the pair's tensor memory
-    // (or its barriers) while the other may still use them (every wait above
-    // is bounded, so all threads get here)
+    // write to its shared memory.  With the sums beside the ring nobody writes
+    // to the others', which signal and go; else the rank-0 CTA signals their
+    // "verdict" barriers, so they stay too: one that gave up waiting for that
+    // signal must not be gone when it comes.  Pairs and multicast: neither CTA
+    // frees the pair's tensor memory (or its barriers) while the other may
+    // still use them (every wait above is bounded, so all threads get here)
     if (cluster_split) {
         cluster_arrive();
-        if (cluster_ctarank() == 0)
+        if (!prm.split_beside || cluster_ctarank() == 0)
             cluster_wait();
     } else if (PAIR || mc > 0) {
         cluster_sync();
@@ -1914,6 +1918,7 @@ struct Plan {
     int kc = 1;                 // k-blocks per pipeline stage
     int rows_per_tile = BM;     // P rows of a CTA's tile (128 or 256)
     size_t ring_bytes = 0;      // bytes of the kernel's TMA ring
+    size_t epi_bytes = 0;       // bytes of its epilogue staging buffers, beside the ring
     size_t ws_floats = 0;       // split-K partials
     size_t ctr_count = 0;       // split-K tile counters
 };
@@ -1998,6 +2003,7 @@ int plan(Params<MAXP>& prm, int max_ctas, Plan* out)
     out->rows_per_tile = BM * MT;
     out->func = reinterpret_cast<const void*>(gemm_fp8_kernel<MAXP, MT, SP, BNC, KC, MX, PAIR>);
     out->ring_bytes = static_cast<size_t>(C::kStages) * C::kStageBytes;
+    out->epi_bytes = static_cast<size_t>(C::kEpiBytes);
     out->grid = grid;
     out->threads = C::kThreads;
     out->smem = C::kSmem;
@@ -2403,6 +2409,7 @@ int build_plan(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int
 {
     const int rc = build_plan_tiles(prm, jobs, bns_in, n, max_ctas, expl, pl);
     prm.cluster_split = 0;
+    prm.split_beside = 0;
     prm.mc = 0;
     if (rc == FP8_OK && pl->cluster == 0 && plan_multicast(prm, jobs, n, pl))
         return rc;
@@ -2426,7 +2433,10 @@ int build_plan(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int
         static_cast<size_t>(s - 1) * P.bn * rows_per_tile * sizeof(float) > pl->ring_bytes ||
         !clusters_fit(*pl, s, prm.total_tiles / s))
         return rc;
+    // (as the kernel sends them: the columns C has, rounded up to 16)
+    const int cols = std::min(P.bn, (P.rows_q + 15) & ~15);
     prm.cluster_split = s;
+    prm.split_beside = static_cast<size_t>(s - 1) * cols * rows_per_tile * sizeof(float) <= pl->epi_bytes;
     pl->cluster = s;
     pl->ws_floats = 0;
     pl->ctr_count = 0;

@@ -118,3 +118,34 @@ def test_stall_switch_counts_launches(gb):
         gb.fp8_test_stall_gemm_loads(0, 0.0)
     assert statuses == [FP8_ERR_TIMEOUT, FP8_ERR_TIMEOUT, 0]
     assert torch.equal(C, ref)
+
+
+@pytest.mark.parametrize("M,N,K,beside", [(16, 4096, 4096, True), (64, 8192, 8192, True), (64, 4096, 8192, False),
+                                          (16, 512, 8192, False)])
+def test_stalled_split_clusters_leave_together(gb, M, N, K, beside):
+    """Slices within a cluster, with the partial sums in the staging buffers
+    (32 KB: the senders leave at once) and in the ring (the senders wait for
+    the rank-0 CTA's signal, and leave with it): every stalled launch ends
+    with the timeout status, however many follow one another, and the next
+    normal one is exact."""
+    plan = gb.gemm_fp8_dense_plan(M, N, K, gb.OUT_F32)
+    assert plan["splits"] > 1 and plan["cluster"] == plan["splits"], plan
+    assert ((plan["splits"] - 1) * M * 128 * 4 <= 32768) == beside, plan
+    run = _dense(gb, M, N, K)
+    ref = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    run(ref)
+    assert gb.fp8_last_device_error() == 0
+    C = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    gb.fp8_test_stall_gemm_loads(3, LIMIT_MS)
+    try:
+        for _ in range(3):
+            run(C)
+        assert gb.fp8_last_device_error() == FP8_ERR_TIMEOUT
+    finally:
+        gb.fp8_test_stall_gemm_loads(0, 0.0)
+    assert torch.isnan(C).all()
+    for _ in range(3):
+        C.fill_(float("nan"))
+        run(C)
+        assert gb.fp8_last_device_error() == 0
+        assert torch.equal(C, ref)
