@@ -916,8 +916,9 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
     // The previous kernel's outputs (operands, scales, the split-K workspace)
     // are read and written by the producer and the epilogue, each of which
     // waits for that kernel itself, the producer with its first stage armed
-    // and its first load the next instruction; the MMA warp reads what the
-    // producer loaded.
+    // and its first load the next instruction.  The MMA warp reads what the
+    // producer loaded; it waits too, so that the limit of its wait for the
+    // first stage does not run while the previous kernel does.
 
     bool cluster_waited = false;                // this thread has waited for the first cluster barrier
     // Roles are chosen per warp; inside warps 0 and 1 only lane 0 works.
@@ -1113,6 +1114,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             bool ok = true;
             // pairs: the even CTA issues the pair's MMAs
             const int mma_tiles = (PAIR && rank != 0) ? 0 : my_tiles;
+            grid_dependency_wait();
             for (int tile = tile0; ok && tile < mma_tiles; tile += tile_step, ++local) {
                 const TileCoord tc = tile == tile0 ? tc_first : tile_coord(prm, tile);
                 const ProblemScalars P = tile == tile0 ? P_first : prm.prob[tc.p];

@@ -149,3 +149,45 @@ def test_stalled_split_clusters_leave_together(gb, M, N, K, beside):
         run(C)
         assert gb.fp8_last_device_error() == 0
         assert torch.equal(C, ref)
+
+
+@pytest.mark.parametrize("kind", ["dense", "pairs", "sparse", "mx", "split cluster"])
+def test_waiting_for_the_previous_kernel_is_no_timeout(gb, kind):
+    """A launch that becomes resident beside the one before it on the stream
+    (a grouped launch capped at two CTAs leaves the other SMs free, and lets
+    its successor in at its start) and then waits for it longer than the limit
+    of the pipeline's waits: that time does not count, the product is whole.
+    The predecessor is 1.1 TFLOP on two CTAs: 16 ms at the nominal rate of two
+    SMs at 2 GHz."""
+    limit_ms = 4.0
+    big_a, big_b = _codes((8192, 8192), 31), _codes((8192, 8192), 32)
+    one = torch.ones(1, device="cuda")
+    big_c = torch.empty((8192, 8192), dtype=torch.bfloat16, device="cuda")
+    big = [gb.make_problem(big_a, big_b, one, 0, one, 0, big_c)]
+    M, N, K = {"dense": (512, 512, 1024), "pairs": (2048, 2048, 4096), "sparse": (512, 512, 1024),
+               "mx": (512, 512, 1024), "split cluster": (16, 2048, 4096)}[kind]
+    if kind == "mx":
+        x, w = torch.randn((M, K), device="cuda"), torch.randn((N, K), device="cuda")
+        (A, sa), (B, sb) = gb.fp8_quantize_mx(x), gb.fp8_quantize_mx(w)
+
+        def run(C):
+            gb.gemm_fp8_mx(A, sa, B, sb, out_dtype=gb.OUT_F32, C=C)
+    else:
+        run = (_sparse if kind == "sparse" else _dense)(gb, M, N, K)
+    ref = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    run(ref)
+    assert gb.fp8_last_device_error() == 0
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    C = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    gb.fp8_test_stall_gemm_loads(0, limit_ms)
+    try:
+        start.record()
+        gb.gemm_fp8_grouped_ex(big, max_ctas=2)
+        run(C)                                  # directly behind it: launched while it runs
+        end.record()
+        assert gb.fp8_last_device_error() == 0
+    finally:
+        gb.fp8_test_stall_gemm_loads(0, 0.0)
+    assert start.elapsed_time(end) > 2 * limit_ms, "the predecessor was too short to show anything"
+    assert torch.equal(C, ref)
