@@ -285,7 +285,10 @@ __device__ __forceinline__ void abort_pipeline(volatile int* flag, int* err)
 // holds the scale of column 32 w + l of window w (0 past the last column).
 // Two windows are kept loaded ahead of use, and the first two are loaded
 // before the epilogue waits for the accumulator, so the scale loads do not
-// add their latency to the epilogue.
+// add their latency to the epilogue.  Ordinary loads, not the read-only path:
+// that one is for data nothing writes while the kernel runs, and the kernel
+// before this one, often the quantiser of these very scales, may still be
+// running when this grid starts.
 struct ScaleWindows {
     float w0, w1;           // the next two windows to hand out
     int next;               // column (from the first) of the window after w1
@@ -294,7 +297,7 @@ struct ScaleWindows {
     __device__ __forceinline__ static float load(const ProblemScalars& P, int j, int lane)
     {
         j += lane;
-        return j < P.rows_q ? __ldg(P.sq + (P.sq_mode ? j : 0)) : 0.0f;
+        return j < P.rows_q ? __ldca(P.sq + (P.sq_mode ? j : 0)) : 0.0f;
     }
     __device__ __forceinline__ void init(const ProblemScalars& P, int jbase, int lane, int cols)
     {
@@ -1339,7 +1342,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             // (pairs: CTA r holds rows 128 r .. of the 256-row tile)
             const int i = PAIR ? tc.m_blk * 2 * BM + BM * static_cast<int>(rank) + row : tc.m_blk * BM * MT + row;
             const bool row_ok = i < P.rows_p;
-            const float fi = row_ok ? __fmul_rn(P.alpha, __ldg(P.sp + (P.sp_mode ? i : 0))) : 0.0f;
+            const float fi = row_ok ? __fmul_rn(P.alpha, __ldca(P.sp + (P.sp_mode ? i : 0))) : 0.0f;
             const int jbase = tc.n_blk * P.bn;
             // every column scale of the tile reaches L1 while its MMAs run:
             // read window by window during the epilogue, each would

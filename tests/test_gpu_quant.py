@@ -232,3 +232,92 @@ def test_tensor_nonfinite_reported(gb, rows, cols, bad):
     gb.fp8_quantize_e4m3(x, 0)
     assert gb.fp8_last_device_error() == -4
     assert gb.fp8_last_device_error() == 0
+
+
+def test_reused_buffers_follow_their_writers(gb):
+    """One code buffer and one scale buffer per kind of quantiser, rewritten
+    on every pass with other values and read by the product right behind (the
+    kernels are launched with programmatic serialization): eager and from a
+    captured graph, every pass equals the calls made one by one.  Covers the
+    per-row, per-tensor (one cluster, and the four-kernel chain), grouped,
+    long-row and block-scaled quantisers, the scale re-layout, and the fused
+    quantise + compress, each before the dense, block-scaled or 2:4 product."""
+    from paper_2602_10262_gb300._lib import FP8QuantJob
+    g = torch.Generator(device="cuda").manual_seed(7)
+    passes, R, K, KL, N = 4, 600, 512, 32896, 512
+
+    def randn(*shape):
+        return torch.randn(shape, generator=g, device="cuda")
+
+    xs = [randn(R, K) * 3.0 ** p for p in range(passes)]
+    longs = [randn(16, KL) * 5.0 ** p for p in range(passes)]
+    W, dW = gb.fp8_quantize_e4m3(randn(N, K), 1)
+    WL, dWL = gb.fp8_quantize_e4m3(randn(N, KL), 1)
+    WX, sWX = gb.fp8_quantize_mx(randn(N, K))
+
+    def codes(rows, cols):
+        return torch.empty((rows, cols), dtype=torch.uint8, device="cuda")
+
+    q, ql, qs = codes(R, K), codes(16, KL), codes(256, K)
+    d, dl, dt = torch.empty(R, device="cuda"), torch.empty(16, device="cuda"), torch.empty(1, device="cuda")
+    v, m = codes(R, K // 2), codes(R, K // 8)
+    sr = codes(R, K // 32)
+    st = torch.empty(gb.fp8_mx_scale_tiled_bytes(R, K), dtype=torch.uint8, device="cuda")
+
+    def outputs():
+        f = lambda r: torch.full((r, N), float("nan"), device="cuda")
+        return [[f(R), f(256), f(R), f(R), f(16), f(R), f(R), f(R)] for _ in range(passes)]
+
+    def grouped(x):
+        job = (FP8QuantJob * 1)(FP8QuantJob(x.data_ptr(), R, K, K, q.data_ptr(), K, d.data_ptr()))
+        stream = torch.cuda.current_stream().cuda_stream
+        assert gb.library().fp8_quantize_e4m3_rows_grouped(job, 1, stream) == 0
+
+    def run(outs, sync=lambda: None):
+        for x, xl, o in zip(xs, longs, outs):
+            for step in (
+                    lambda: gb.fp8_quantize_e4m3(x, 1, q=q, dequant_scale=d),
+                    lambda: gb.gemm_fp8_dense(q, W, d, 1, dW, 1, 1.0, gb.OUT_F32, C=o[0]),
+                    lambda: gb.fp8_quantize_e4m3(x[:256], 0, q=qs, dequant_scale=dt),
+                    lambda: gb.gemm_fp8_dense(qs, W, dt, 0, dW, 1, 1.0, gb.OUT_F32, C=o[1]),
+                    lambda: gb.fp8_quantize_e4m3(x, 0, q=q, dequant_scale=dt),
+                    lambda: gb.gemm_fp8_dense(q, W, dt, 0, dW, 1, 1.0, gb.OUT_F32, C=o[2]),
+                    lambda: grouped(x),
+                    lambda: gb.gemm_fp8_dense(W, q, dW, 1, d, 1, 1.0, gb.OUT_F32, C=o[3].view(N, R)),
+                    lambda: gb.fp8_quantize_e4m3(xl, 1, q=ql, dequant_scale=dl),
+                    lambda: gb.gemm_fp8_dense(ql, WL, dl, 1, dWL, 1, 1.0, gb.OUT_F32, C=o[4]),
+                    lambda: gb.fp8_quantize_mx(x, q=q, scales=st),
+                    lambda: gb.gemm_fp8_mx(q, st, WX, sWX, out_dtype=gb.OUT_F32, C=o[5]),
+                    lambda: gb.fp8_quantize_mx(x, scale_layout=0, q=q, scales=sr),
+                    lambda: gb.fp8_mx_scales_to_tiled(sr, R, K, st),
+                    lambda: gb.gemm_fp8_mx(q, st, WX, sWX, out_dtype=gb.OUT_F32, C=o[6]),
+                    lambda: gb.fp8_quantize_e4m3_prune24(x, q=q, dequant_scale=d, a_vals=v, a_meta=m),
+                    lambda: gb.gemm_fp8_sparse24(v, m, W, d, 1, dW, 1, 1.0, gb.OUT_F32, C=o[7])):
+                step()
+                sync()
+
+    want = outputs()
+    run(want, torch.cuda.synchronize)
+    assert not any(torch.isnan(t).any() for o in want for t in o)
+    assert torch.equal(want[0][5], want[0][6])
+    assert not torch.equal(want[0][0], want[1][0])
+
+    def check(outs):
+        for a, b in zip(outs, want):
+            assert all(torch.equal(s, t) for s, t in zip(a, b))
+
+    for _ in range(3):
+        got = outputs()
+        run(got)
+        check(got)
+    got = outputs()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(got)
+    for _ in range(3):
+        for o in got:
+            for t in o:
+                t.fill_(float("nan"))
+        graph.replay()
+        check(got)
+    assert gb.fp8_last_device_error() == 0
