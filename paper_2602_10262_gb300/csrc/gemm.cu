@@ -1741,6 +1741,7 @@ struct Job {
     int fmt_p, fmt_q;       // fp8_format of P and Q (instruction-descriptor A / B format)
     const uint8_t* sfp;     // block-scaled problems: tiled E8M0 scales of P and Q
     const uint8_t* sfq;     // (nullptr otherwise)
+    int max_splits = 0;     // > 0: k-slices per tile at most (see build_plan)
 };
 
 bool valid_format(int f)
@@ -1809,6 +1810,26 @@ int slice_kblocks(int k_blocks, int s)
     return ((k_blocks + s - 1) / s + 3) / 4 * 4;
 }
 
+// Columns of a tile's partial sums as cluster split-K sends them: those C
+// has, rounded up to 16.
+int64_t split_columns(int64_t rows_q, int bn)
+{
+    return std::min<int64_t>(bn, (rows_q + 15) / 16 * 16);
+}
+
+// Slices of a block-scaled product's tile (one column of tiles, 128 rows)
+// whose partial sums the TMA ring of one CTA receives: gemm_fp8_mx promises
+// to need no workspace, so it never splits further.  128 columns: 4 slices,
+// 96: 5, 64: 7, 48 and fewer: 8.
+int mx_ring_splits(int64_t rows_q)
+{
+    const auto ring = [](auto cfg) { return int64_t{decltype(cfg)::kStages} * decltype(cfg)::kStageBytes; };
+    const int64_t bytes = rows_q <= 16   ? ring(Cfg<1, false, 16, 2, 1>{})
+                          : rows_q <= 64 ? ring(Cfg<1, false, 64, 2, 1>{})
+                                         : ring(Cfg<1, false, 128, 2, 1>{});
+    return static_cast<int>(1 + bytes / (split_columns(rows_q, 128) * BM * static_cast<int64_t>(sizeof(float))));
+}
+
 int split_count(const Job& j)
 {
     const int sms = sm_count();
@@ -1825,6 +1846,10 @@ int split_count(const Job& j)
     const int k_blocks = static_cast<int>((j.K + BK - 1) / BK);
     int s = std::min<int64_t>(8, sms / tiles);
     s = std::min(s, k_blocks / 8);
+    if (j.sfp)
+        s = std::min(s, mx_ring_splits(j.rows_q));
+    if (j.max_splits > 0)
+        s = std::min(s, j.max_splits);
     if (s <= 1)
         return 1;
     const int kbs = slice_kblocks(k_blocks, s);
@@ -2409,8 +2434,8 @@ bool plan_multicast(Params<MAXP>& prm, const Job* jobs, int n, Plan* pl)
 // problem, the other slices' partial sums fit in a CTA's TMA ring, and all
 // clusters can be resident at once; otherwise the global split path.
 template <int MAXP>
-int build_plan(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int max_ctas,
-               const TileChoice* expl, Plan* pl, bool allow_cluster = false)
+int build_plan_form(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int max_ctas,
+                    const TileChoice* expl, Plan* pl, bool allow_cluster)
 {
     const int rc = build_plan_tiles(prm, jobs, bns_in, n, max_ctas, expl, pl);
     prm.cluster_split = 0;
@@ -2434,17 +2459,33 @@ int build_plan(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int
     const ProblemScalars& P = prm.prob[0];
     const int s = P.splits;
     const size_t rows_per_tile = static_cast<size_t>(pl->rows_per_tile);
-    if (s < 2 || s > 8 || pl->grid != prm.total_tiles || prm.total_tiles % s != 0 ||
-        static_cast<size_t>(s - 1) * P.bn * rows_per_tile * sizeof(float) > pl->ring_bytes ||
+    const size_t received = static_cast<size_t>(s - 1) * split_columns(P.rows_q, P.bn) * rows_per_tile * sizeof(float);
+    if (s < 2 || s > 8 || pl->grid != prm.total_tiles || prm.total_tiles % s != 0 || received > pl->ring_bytes ||
         !clusters_fit(*pl, s, prm.total_tiles / s))
         return rc;
-    // (as the kernel sends them: the columns C has, rounded up to 16)
-    const int cols = std::min(P.bn, (P.rows_q + 15) & ~15);
     prm.cluster_split = s;
-    prm.split_beside = static_cast<size_t>(s - 1) * cols * rows_per_tile * sizeof(float) <= pl->epi_bytes;
+    prm.split_beside = received <= pl->epi_bytes;
     pl->cluster = s;
     pl->ws_floats = 0;
     pl->ctr_count = 0;
+    return rc;
+}
+
+// As above; a block-scaled product, which has no workspace (gemm_fp8_mx's
+// contract), takes the most slices whose clusters can all be resident at once,
+// down to none (19 tiles: 19 clusters of eight do not fit).
+template <int MAXP>
+int build_plan(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int n, int max_ctas,
+               const TileChoice* expl, Plan* pl, bool allow_cluster = false)
+{
+    int rc = build_plan_form(prm, jobs, bns_in, n, max_ctas, expl, pl, allow_cluster);
+    if (n != 1 || jobs[0].sfp == nullptr)
+        return rc;
+    Job j = jobs[0];
+    while (rc == FP8_OK && workspace_bytes(*pl) != 0) {
+        j.max_splits = prm.prob[0].splits - 1;
+        rc = build_plan_form(prm, &j, bns_in, n, max_ctas, expl, pl, allow_cluster);
+    }
     return rc;
 }
 

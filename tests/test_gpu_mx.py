@@ -407,3 +407,25 @@ def test_mx_quantize_alignments(gb, orc, layout, rows, cols):
         assert np.array_equal(s.cpu().numpy(), want)
         assert bool((qb[qoff:].view(rows, cols + qpad)[:, cols:] == 0xA5).all())
     assert gb.fp8_last_device_error() == 0
+
+
+# rows: one column of tiles of each width, odd ones among them; N: few tiles
+# in many slices, as many clusters of eight as there are SMs / 8, and more
+# than fit; K from the first split length up
+@pytest.mark.parametrize("M", [1, 16, 17, 33, 48, 64, 70, 96, 100, 127, 128])
+def test_mx_needs_no_workspace(gb, M):
+    """gemm_fp8_mx promises to need none: a product split along K adds its
+    slices up within clusters, whatever its size."""
+    for N in (129, 256, 777, 1024, 2048, 2176, 2304, 2432, 3000, 4096, 8192, 9728, 14336):
+        for K in (4096, 4128, 8192, 14336, 16384, 32768):
+            plan = gb.gemm_fp8_mx_plan(M, N, K)
+            assert plan["workspace_bytes"] == 0, (N, K, plan)
+            assert plan["splits"] == 1 or plan["cluster"] == plan["splits"], (N, K, plan)
+
+
+@pytest.mark.parametrize("out", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(128, 1024, 8192), (128, 2048, 8192), (64, 2048, 8192), (96, 2048, 14336),
+                                   (70, 1024, 8192), (48, 2432, 8192), (16, 2432, 8192)])
+def test_mx_few_tiles_split_exact(gb, M, N, K, out):
+    assert gb.gemm_fp8_mx_plan(M, N, K, out)["splits"] > 1
+    _check_mx_exact(gb, M, N, K, out)
