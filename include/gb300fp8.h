@@ -431,6 +431,8 @@ int fp8_gemm_set_tile_config(int mt, int group_m);
  * raster divide into such clusters: each CTA loads its own A rows (MMA-M
  * side) and a quarter (half) of the shared B block (MMA-N side), multicast
  * to the cluster by TMA, which cuts the bytes each SM reads per k-block.
+ * Only in a process that sees one GPU and is no rank of a larger job (the
+ * environment's WORLD_SIZE above 1): elsewhere mode 1 is as 0.
  * mode 0 (default): never; measured 2-9 % slower on mid-size and skinny
  * products on GB300.  Results do not depend on it.  FP8_ERR_INVALID for any
  * other mode.  Affects launches planned after the call, from any thread. */

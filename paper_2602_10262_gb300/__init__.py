@@ -193,7 +193,7 @@ def fp8_gemm_set_tile_config(mt: int = 0, group_m: int = 0) -> None:
 
 def fp8_gemm_set_multicast(mode: int = 0) -> None:
     """B-block multicast within clusters of 128-row-tile launches: 1 where it
-    applies, 0 never (default)."""
+    applies (a process with one GPU, no rank of a larger job), 0 never (default)."""
     _check(library().fp8_gemm_set_multicast(int(mode)), "fp8_gemm_set_multicast")
 
 

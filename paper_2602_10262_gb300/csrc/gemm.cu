@@ -2390,6 +2390,22 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
 // applies, 0 = never (default: measured slower, see plan_multicast).
 std::atomic<int> g_multicast_mode{0};
 
+// Whether this process works with one GPU alone: it sees no other, and is no
+// rank of a larger job.  Looked at once.
+bool lone_gpu_process()
+{
+    static const bool lone = [] {
+        int devices = 0;
+        if (cudaGetDeviceCount(&devices) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        const char* ranks = std::getenv("WORLD_SIZE");
+        return devices == 1 && (!ranks || std::atoi(ranks) <= 1);
+    }();
+    return lone;
+}
+
 // Q multicast for a launch of 128-row tiles of one dense problem that is not
 // split along K: clusters of mc CTAs (4, else 2) take mc consecutive tiles of
 // the raster, i.e. mc row blocks of one N column, and each loads 1/mc of the
@@ -2399,7 +2415,8 @@ std::atomic<int> g_multicast_mode{0};
 // walks the same columns in lockstep), the Q slices stay whole swizzle atoms
 // (8 rows), and every cluster can be resident at once.  Remakes the Q map
 // for the slice box; the MMAs and their order do not change, so neither do
-// the results.  Off unless enabled: on GB300 it made every shape it applies
+// the results.  Never in a job of several GPUs, where no multicast load may
+// run beside memory that other GPUs share.  Off unless enabled: on GB300 it made every shape it applies
 // to slower (1024^3 by 9 %, 2048^3 by 7 %, 128 x 8192 x 8192 by 2 %, one
 // box, interleaved replays): each SM reads fewer B bytes, but the k-loops
 // here are not bound by them, and the clusters' lockstep ring and launch
@@ -2408,7 +2425,7 @@ template <int MAXP>
 bool plan_multicast(Params<MAXP>& prm, const Job* jobs, int n, Plan* pl)
 {
     if (g_multicast_mode.load(std::memory_order_relaxed) != 1 || n != 1 || pl->rows_per_tile != BM ||
-        jobs[0].E != nullptr || jobs[0].sfp != nullptr)
+        jobs[0].E != nullptr || jobs[0].sfp != nullptr || !lone_gpu_process())
         return false;
     Problem& P = prm.prob[0];
     if (P.splits != 1)

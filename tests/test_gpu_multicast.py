@@ -139,3 +139,14 @@ def test_multicast_off_by_default(gb):
                        cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0, r.stderr
     assert r.stdout.strip() == "0"
+
+
+def test_multicast_never_in_a_job_of_several_ranks(gb):
+    """Switched on in a process that is one rank of two: planned nowhere."""
+    code = ("import paper_2602_10262_gb300 as gb; gb.library(); gb.fp8_gemm_set_multicast(1); "
+            "print(gb.gemm_fp8_dense_plan(1024, 1024, 1024)['multicast'])")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                       env=dict(os.environ, WORLD_SIZE="2"))
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.strip() == "0"
