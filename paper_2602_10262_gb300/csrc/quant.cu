@@ -108,8 +108,13 @@ __device__ __forceinline__ void scale_from_amax(uint32_t amax_bits, float& s, fl
 // TPR threads (a warp, or a whole number of warps of one block) take a row,
 // each holding U vectors of W consecutive elements: vector u of thread t
 // starts at column (u * TPR + t) * W.  W = 8 is one 32-byte load a vector
-// (x 32-aligned, ldx % 8 == 0), W = 4 one 16-byte load, or guarded scalar
-// loads where x allows neither and past the last whole vector.
+// (x 32-aligned, ldx % 8 == 0) or two 16-byte ones, with guarded scalar loads
+// past the last whole vector.  W = 1, where x or q allows neither, keeps a
+// warp's scalar loads and byte stores side by side: 4096 x 14336 at odd
+// offsets 49.9 us (four consecutive elements a thread 94.6, the row read twice
+// 86.2; 43.5 aligned).  Two 16-byte loads a vector, not vectors of four: half
+// as many addresses and guards, and the registers that they took left one
+// block an SM (the same size at 16-byte offsets 64.3 -> 45.6 us).
 //
 // What bounds it: HBM, once enough bytes are in flight.  Rows are loaded
 // once instead of twice (the second pass over L2 cost issue slots and load
@@ -136,29 +141,23 @@ constexpr int row_block()
     return TPR > kRowBlock ? TPR : kRowBlock;
 }
 
-// W consecutive floats at p, the first `left` of them inside the row (0 for
+// 8 consecutive floats at p, the first `left` of them inside the row (0 for
 // the others).  vec: p is aligned for whole-vector loads.
-template <int W>
-__device__ __forceinline__ void load_vec(const float* p, int64_t left, bool vec, float (&v)[W])
+__device__ __forceinline__ void load_vec8(const float* p, int64_t left, bool vec, float (&v)[8])
 {
-    if (vec && left >= W) {
-        if constexpr (W == 8) {
-            asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
-                           "=f"(v[7])
-                         : "l"(p));
-        } else {
-            const float4 a = __ldca(reinterpret_cast<const float4*>(p));
-            v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
-        }
+    if (vec && left >= 8) {
+        asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+                       "=f"(v[7])
+                     : "l"(p));
     } else {
 #pragma unroll
-        for (int i = 0; i < W; ++i)
+        for (int i = 0; i < 8; ++i)
             v[i] = i < left ? __ldca(p + i) : 0.0f;
     }
 }
 
-// As load_vec<8> for rows that are only 16-byte aligned (left is 0 or >= 8).
+// As load_vec8 for rows that are only 16-byte aligned (left is 0 or >= 8).
 __device__ __forceinline__ void load_two_vec4(const float* p, int64_t left, float (&v)[8])
 {
     const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -166,6 +165,18 @@ __device__ __forceinline__ void load_two_vec4(const float* p, int64_t left, floa
     const float4 b = left > 0 ? __ldca(reinterpret_cast<const float4*>(p) + 1) : z;
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
     v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+}
+
+// 8 elements at p, the first `left` inside the row.  xa: alignment of the
+// rows in elements (8, 4 or 1).
+__device__ __forceinline__ void load_8(const float* p, int64_t left, int xa, float (&v)[8])
+{
+    if (xa == 8 || left < 8)
+        load_vec8(p, left, xa == 8, v);
+    else if (xa == 4)
+        load_two_vec4(p, left, v);
+    else
+        load_vec8(p, left, false, v);
 }
 
 // Max over the TPR threads of a row group.  red: one entry per warp of the
@@ -204,44 +215,49 @@ __device__ __forceinline__ uint32_t enc4(const float* v, float s)
     return enc4<FMT>(make_float4(v[0], v[1], v[2], v[3]), s);
 }
 
-// The codes of one vector to qr (qa: the row's store alignment, 8, 4 or 1).
-template <int FMT, int W>
-__device__ __forceinline__ void store_codes(uint8_t* qr, int64_t left, int qa, const float (&v)[W], float s)
+// The codes of 8 elements to qr, the first `left` inside the row (qa: the
+// row's store alignment, 8, 4 or 1).
+template <int FMT>
+__device__ __forceinline__ void store_codes8(uint8_t* qr, int64_t left, int qa, const float (&v)[8], float s)
 {
     if (left <= 0)
         return;
-    uint32_t w[W / 4];
-#pragma unroll
-    for (int h = 0; h < W / 4; ++h)
-        w[h] = enc4<FMT>(v + 4 * h, s);
-    if (left >= W && qa >= W) {
-        if constexpr (W == 8)
-            *reinterpret_cast<uint2*>(qr) = make_uint2(w[0], w[1]);
-        else
-            *reinterpret_cast<uint32_t*>(qr) = w[0];
-    } else if (left >= W && qa >= 4) {
-#pragma unroll
-        for (int h = 0; h < W / 4; ++h)
-            reinterpret_cast<uint32_t*>(qr)[h] = w[h];
+    const uint32_t w[2] = {enc4<FMT>(v, s), enc4<FMT>(v + 4, s)};
+    if (left >= 8 && qa >= 8) {
+        *reinterpret_cast<uint2*>(qr) = make_uint2(w[0], w[1]);
+    } else if (left >= 8 && qa >= 4) {
+        reinterpret_cast<uint32_t*>(qr)[0] = w[0];
+        reinterpret_cast<uint32_t*>(qr)[1] = w[1];
     } else {
 #pragma unroll
-        for (int i = 0; i < W; ++i)
+        for (int i = 0; i < 8; ++i)
             if (i < left)
                 qr[i] = static_cast<uint8_t>(w[i / 4] >> (8 * (i % 4)));
     }
 }
 
+template <int FMT>
+__device__ __forceinline__ uint8_t enc1(float v, float s)
+{
+    return static_cast<uint8_t>(enc2<FMT>(__fmul_rn(v, s), 0.0f) & 0xFFu);
+}
+
 // One row by its TPR threads (t: index within them; ok: the row exists).
+// xa, qa: alignment of the rows of x and q in elements (8, 4 or 1).
 template <int FMT, int TPR, int U, int W>
-__device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols, uint8_t* qr, float* d_out, bool vec,
+__device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols, uint8_t* qr, float* d_out, int xa,
                                                   int qa, int* err, uint32_t* red, int t, bool ok)
 {
+    static_assert(W == 8 || W == 1, "whole vectors or single elements");
     float v[U][W];
     const int64_t n = ok ? cols : 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
-        load_vec<W>(xr + c, n - c, vec, v[u]);
+        if constexpr (W == 8)
+            load_8(xr + c, n - c, xa, v[u]);
+        else
+            v[u][0] = c < n ? __ldca(xr + c) : 0.0f;
     }
     const uint32_t m = row_max<TPR>(held_amax(v), red);
     float s, dq;
@@ -254,7 +270,10 @@ __device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols,
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
-        store_codes<FMT, W>(qr + c, n - c, qa, v[u], s);
+        if constexpr (W == 8)
+            store_codes8<FMT>(qr + c, n - c, qa, v[u], s);
+        else if (c < n)
+            qr[c] = enc1<FMT>(v[u][0], s);
     }
 }
 
@@ -262,7 +281,7 @@ template <int FMT, int TPR, int U, int W>
 __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float* __restrict__ x, int64_t rows,
                                                                      int64_t cols, int64_t ldx,
                                                                      uint8_t* __restrict__ q, int64_t ldq,
-                                                                     float* __restrict__ d, int vec, int qa,
+                                                                     float* __restrict__ d, int xa, int qa,
                                                                      int early, int* err)
 {
     grid_launch_dependents();
@@ -287,7 +306,7 @@ __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float
     for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRows; r0 < rows;
          r0 += static_cast<int64_t>(gridDim.x) * kRows, flip ^= 1) {
         const int64_t r = r0 + threadIdx.x / TPR;
-        quantize_held_row<FMT, TPR, U, W>(x + r * ldx, cols, q + r * ldq, d + r, vec != 0, qa, err, red[flip], t,
+        quantize_held_row<FMT, TPR, U, W>(x + r * ldx, cols, q + r * ldq, d + r, xa, qa, err, red[flip], t,
                                           r < rows);
     }
 }
@@ -329,7 +348,7 @@ __global__ void __launch_bounds__(row_block<TPR>()) quant_row_prune_kernel(const
         for (int u = 0; u < U; ++u) {
             const int64_t c = static_cast<int64_t>(u * TPR + t) * 8;
             if (wide)
-                load_vec<8>(xr + c, n - c, true, v[u]);
+                load_vec8(xr + c, n - c, true, v[u]);
             else
                 load_two_vec4(xr + c, n - c, v[u]);
         }
@@ -403,7 +422,7 @@ __device__ __forceinline__ void quantize_row(const float* __restrict__ xr, int64
         reinterpret_cast<uint32_t*>(qr)[i] = enc4<FMT>(v, s);
     }
     for (int64_t c = nvec * 4 + threadIdx.x; c < cols; c += kThreads)
-        qr[c] = static_cast<uint8_t>(enc2<FMT>(__fmul_rn(xr[c], s), 0.0f) & 0xFFu);
+        qr[c] = enc1<FMT>(xr[c], s);
 }
 
 template <int FMT>
@@ -471,8 +490,8 @@ __global__ void __launch_bounds__(kThreads) quant_long_row_prune_kernel(const fl
 struct RowJobs {
     fp8_quant_job job[FP8_QUANT_GROUPED_MAX];
     int64_t row_start[FP8_QUANT_GROUPED_MAX + 1];
-    int vec[FP8_QUANT_GROUPED_MAX];       // whole-vector loads of the launch's W (or, read twice, of 4)
-    int qa[FP8_QUANT_GROUPED_MAX];        // store alignment of the codes: 8, 4 or 1
+    int xa[FP8_QUANT_GROUPED_MAX];        // alignment of the rows of x and of the codes, in elements: 8, 4 or 1
+    int qa[FP8_QUANT_GROUPED_MAX];
     int n;
 };
 
@@ -500,7 +519,7 @@ __global__ void __launch_bounds__(kGroupedTpr) quant_rows_grouped_kernel(const _
         const fp8_quant_job& J = jobs.job[j];
         const int64_t r = g - jobs.row_start[j];
         quantize_held_row<0, kGroupedTpr, U, W>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r,
-                                                jobs.vec[j] != 0, jobs.qa[j], err, red[flip], threadIdx.x, true);
+                                                jobs.xa[j], jobs.qa[j], err, red[flip], threadIdx.x, true);
     }
 }
 
@@ -514,7 +533,7 @@ __global__ void __launch_bounds__(kThreads) quant_long_rows_grouped_kernel(const
         const int j = job_of_row(jobs, g);
         const fp8_quant_job& J = jobs.job[j];
         const int64_t r = g - jobs.row_start[j];
-        quantize_row<0>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r, jobs.vec[j] && jobs.qa[j] >= 4,
+        quantize_row<0>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r, jobs.xa[j] >= 4 && jobs.qa[j] >= 4,
                         err, red);
     }
 }
@@ -523,18 +542,6 @@ __global__ void __launch_bounds__(kThreads) quant_long_rows_grouped_kernel(const
 //
 // A matrix is cut into vectors of 8 consecutive elements of a row, ceil(cols
 // / 8) per row; a contiguous matrix comes as one long row.
-
-// 8 elements at p, the first `left` inside the row.  xa: alignment of the
-// rows in elements (8, 4 or 1).
-__device__ __forceinline__ void load_8(const float* p, int64_t left, int xa, float (&v)[8])
-{
-    if (xa == 8 || left < 8)
-        load_vec<8>(p, left, xa == 8, v);
-    else if (xa == 4)
-        load_two_vec4(p, left, v);
-    else
-        load_vec<8>(p, left, false, v);
-}
 
 // Whole tensor in one cluster: thread t of CTA c holds vectors (u * kCtas + c)
 // * kClusterThreads + t.  What bounds it is latency: one launch, one load
@@ -585,7 +592,7 @@ __global__ void __launch_bounds__(kClusterThreads) quant_cluster_kernel(const fl
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-        store_codes<FMT, 8>(q + r[u] * ldq + c[u], r[u] < rows ? cols - c[u] : 0, qa, v[u], s);
+        store_codes8<FMT>(q + r[u] * ldq + c[u], r[u] < rows ? cols - c[u] : 0, qa, v[u], s);
     cluster_sync();                        // no CTA leaves while a peer may read its maximum
 }
 
@@ -676,7 +683,7 @@ __global__ void __launch_bounds__(kThreads) quant_encode_kernel(const float* __r
         }
 #pragma unroll
         for (int k = 0; k < kItems; ++k)
-            store_codes<FMT, 8>(q + r[k] * ldq + c[k], left[k], qa, v[k], s);
+            store_codes8<FMT>(q + r[k] * ldq + c[k], left[k], qa, v[k], s);
     }
 }
 
@@ -787,12 +794,12 @@ struct RowLaunch {
     {
         const int xa = row_align(x, ldx, 4), qa = row_align(q, ldq, 1);
         const int grid = row_grid(rows, row_block<TPR>() / TPR);
-        if (xa == 8)
+        if (xa >= 4 && qa >= 4)
             launch_dependent(quant_row_kernel<FMT, TPR, U, 8>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q, ldq,
-                             d, 1, qa, rows <= 2 * sm_count(), err);
+                             d, xa, qa, rows <= 2 * sm_count(), err);
         else
-            launch_dependent(quant_row_kernel<FMT, TPR, 2 * U, 4>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q,
-                             ldq, d, xa == 4, qa, rows <= 2 * sm_count(), err);
+            launch_dependent(quant_row_kernel<FMT, TPR, 8 * U, 1>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q,
+                             ldq, d, xa, qa, rows <= 2 * sm_count(), err);
     }
 };
 
@@ -962,7 +969,7 @@ __global__ void __launch_bounds__(kThreads) quant_mx_kernel(const float* __restr
             code = static_cast<uint32_t>(e + 127);
             s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);     // 2^-e, normal
         }
-        store_codes<FMT, 8>(q + r * ldq + c, in ? 8 : 0, qa, v, s);
+        store_codes8<FMT>(q + r * ldq + c, in ? 8 : 0, qa, v, s);
         // blocks past cols and padding rows: scale 1
         uint32_t word = (in ? code : 127u) << (8 * ((lane >> 2) & 3));
         word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
@@ -1167,9 +1174,9 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
         const int k = rj.n++;
         rj.job[k] = J;
         rj.row_start[k] = rows;
-        rj.vec[k] = row_align(J.x, J.ldx, 4);
+        rj.xa[k] = row_align(J.x, J.ldx, 4);
         rj.qa[k] = row_align(J.q, J.ldq, 1);
-        wide = wide && rj.vec[k] == 8;
+        wide = wide && rj.xa[k] >= 4 && rj.qa[k] >= 4;
         max_cols = std::max(max_cols, J.cols);
         rows += J.rows;
     }
@@ -1178,23 +1185,21 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
         return FP8_OK;
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
-    for (int i = 0; i < rj.n; ++i)
-        rj.vec[i] = rj.vec[i] >= 4;               // a row of the launch's W (wide: all 8) or of 4
     const int grid = row_grid(rows, 1);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     int* err = device_error_word();
-    const auto launch = [&](auto* w8, auto* w4) {
+    const auto launch = [&](auto* w8, auto* w1) {
         if (wide)
             launch_dependent(w8, grid, kGroupedTpr, st, rj, err);
         else
-            launch_dependent(w4, grid, kGroupedTpr, st, rj, err);
+            launch_dependent(w1, grid, kGroupedTpr, st, rj, err);
     };
     if (max_cols <= 8 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<1, 8>, quant_rows_grouped_kernel<2, 4>);
+        launch(quant_rows_grouped_kernel<1, 8>, quant_rows_grouped_kernel<8, 1>);
     else if (max_cols <= 16 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<2, 8>, quant_rows_grouped_kernel<4, 4>);
+        launch(quant_rows_grouped_kernel<2, 8>, quant_rows_grouped_kernel<16, 1>);
     else if (max_cols <= 32 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<4, 8>, quant_rows_grouped_kernel<8, 4>);
+        launch(quant_rows_grouped_kernel<4, 8>, quant_rows_grouped_kernel<32, 1>);
     else
         quant_long_rows_grouped_kernel<<<grid, kThreads, 0, st>>>(rj, err);
     GB_CUDA_OK(cudaGetLastError());

@@ -321,3 +321,30 @@ def test_reused_buffers_follow_their_writers(gb):
         graph.replay()
         check(got)
     assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("rows,cols", [(r, c) for r in (3, 401) for c in
+                                       (1, 33, 255, 512, 1024, 1031, 4096, 4100, 6144, 12288, 14336, 16384, 32768)])
+def test_row_mixed_alignments(gb, orc, rows, cols):
+    """x and q of different alignment (either may rule the whole vectors
+    out), by the single call and by the grouped one."""
+    from paper_2602_10262_gb300._lib import FP8QuantJob
+    x = workloads.randn_f32((rows, cols), seed=rows + cols)
+    x[rows - 1, cols - 1] = 3e4
+    qo, do = orc.quantize(x, 1)
+    for pad, off, qpad, qoff in ((-cols % 8, 0, 1 - cols % 2, 1), (-cols % 8, 4, -cols % 16, 4),
+                                 (1 - cols % 2, 0, -cols % 8, 0), (-cols % 4, 4, 3, 2)):
+        xt = torch.zeros(rows * (cols + pad) + off, device="cuda")[off:].view(rows, cols + pad)[:, :cols]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((rows * (cols + qpad) + qoff,), 0xA5, dtype=torch.uint8, device="cuda")
+        qt = qb[qoff:].view(rows, cols + qpad)[:, :cols]
+        d = torch.empty(rows, device="cuda")
+        gb.fp8_quantize_e4m3(xt, 1, q=qt, dequant_scale=d)
+        single = qb.clone()
+        assert np.array_equal(qt.cpu().numpy(), qo) and np.array_equal(d.cpu().numpy(), do)
+        qb.fill_(0xA5), d.zero_()
+        job = (FP8QuantJob * 1)(FP8QuantJob(xt.data_ptr(), rows, cols, xt.stride(0), qt.data_ptr(), qt.stride(0),
+                                            d.data_ptr()))
+        assert gb.library().fp8_quantize_e4m3_rows_grouped(job, 1, torch.cuda.current_stream().cuda_stream) == 0
+        assert torch.equal(qb, single) and np.array_equal(d.cpu().numpy(), do)
+    assert gb.fp8_last_device_error() == 0
