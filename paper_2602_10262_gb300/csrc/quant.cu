@@ -906,6 +906,21 @@ __device__ __forceinline__ int64_t mx_tiled_offset(int64_t r, int64_t b, int64_t
     return 512 * ((r >> 7) * kb + (b >> 2)) + 16 * (r & 31) + 4 * ((r & 127) >> 5) + (b & 3);
 }
 
+// Scale code of a block and its encoding scale 2^-e from the block's amax bits
+// (see quant_mx_kernel; 0 and 1 where amax is 0 or not finite).
+template <int FMT>
+__device__ __forceinline__ uint32_t mx_block_scale(uint32_t m, float& s)
+{
+    constexpr int kEmax = FMT == 1 ? 15 : 8;
+    s = 1.0f;
+    if (m == 0u || m >= kInfBits)
+        return 0u;
+    const int E = static_cast<int>(m >> 23);      // biased exponent of amax
+    const int e = E == 0 ? -127 : max(E - 127 - kEmax, -127);
+    s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);         // normal
+    return static_cast<uint32_t>(e + 127);
+}
+
 // One warp quantises a 256-column window of one row at a time: lane l holds
 // columns 8l .. 8l + 7, so a 32-element block is four lanes, and its amax is
 // their local maxima and two shuffles.  For a non-zero block, e = floor(log2
@@ -925,7 +940,13 @@ __device__ __forceinline__ int64_t mx_tiled_offset(int64_t r, int64_t b, int64_t
 // 46.5; 16384 x 8192 112, 103; 16 x 4096 3.6, 2.0).  Two, four or eight
 // windows a warp at once, loads first, were slower (16.7, 17.6 and 23.9 us at
 // 4096 x 4096): enough warps have a load in flight.
-template <int FMT, int TILED>
+// WIDE = false, where the rows of x or q start on any element: lane l holds
+// columns l, l + 32, ..., one of each block, so that loads and byte stores lie
+// side by side and a block's amax is one warp reduction; lane k takes the
+// scale of block k (16384 x 4096 at odd offsets with tiled scales: 72.5 us,
+// eight consecutive elements a lane 92.1, four 74.3; each lane taking all
+// eight scales 94.8).
+template <int FMT, int TILED, bool WIDE>
 __global__ void __launch_bounds__(kThreads) quant_mx_kernel(const float* __restrict__ x, int64_t rows,
                                                             int64_t cols, int64_t ldx, int xa,
                                                             uint8_t* __restrict__ q, int64_t ldq, int qa,
@@ -933,7 +954,6 @@ __global__ void __launch_bounds__(kThreads) quant_mx_kernel(const float* __restr
 {
     grid_launch_dependents();
     grid_dependency_wait();
-    constexpr int kEmax = FMT == 1 ? 15 : 8;
     const int lane = threadIdx.x & 31;
     const int64_t kb = (cols + 127) / 128;
     const int64_t segs = (cols + 255) / 256;
@@ -949,31 +969,59 @@ __global__ void __launch_bounds__(kThreads) quant_mx_kernel(const float* __restr
             r = i / segs;
             seg = i - r * segs;
         }
-        const int64_t c = seg * 256 + 8 * lane;
-        const bool in = c < cols && r < rows;     // cols % 32 == 0: a lane's eight columns are all in or out
-        float v[8];
-        load_8(x + r * ldx + c, in ? 8 : 0, xa, v);
-        uint32_t m = 0;
+        uint32_t word;                            // the four scale codes of this half warp's k-block
+        if constexpr (WIDE) {
+            const int64_t c = seg * 256 + 8 * lane;
+            const bool in = c < cols && r < rows; // cols % 32 == 0: a lane's eight columns are all in or out
+            float v[8];
+            load_8(x + r * ldx + c, in ? 8 : 0, xa, v);
+            uint32_t m = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            m = max(m, abs_bits(v[k]));
-        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-        if (m >= kInfBits && (lane & 3) == 0)
-            report_device_error(err, FP8_ERR_NONFINITE);
-        uint32_t code = 0;
-        float s = 1.0f;
-        if (m != 0u && m < kInfBits) {
-            const int E = static_cast<int>(m >> 23);  // biased exponent of amax
-            const int e = E == 0 ? -127 : max(E - 127 - kEmax, -127);
-            code = static_cast<uint32_t>(e + 127);
-            s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);     // 2^-e, normal
+            for (int k = 0; k < 8; ++k)
+                m = max(m, abs_bits(v[k]));
+            m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+            m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+            if (m >= kInfBits && (lane & 3) == 0)
+                report_device_error(err, FP8_ERR_NONFINITE);
+            float s;
+            const uint32_t code = mx_block_scale<FMT>(m, s);
+            store_codes8<FMT>(q + r * ldq + c, in ? 8 : 0, qa, v, s);
+            // blocks past cols and padding rows: scale 1
+            word = (in ? code : 127u) << (8 * ((lane >> 2) & 3));
+            word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
+            word |= __shfl_xor_sync(0xFFFFFFFFu, word, 8);
+        } else {
+            // blocks of this window inside the matrix
+            const int nb = r < rows ? static_cast<int>(min(cols - seg * 256, static_cast<int64_t>(256))) / 32 : 0;
+            const float* xw = x + r * ldx + seg * 256 + lane;
+            uint8_t* qw = q + r * ldq + seg * 256 + lane;
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                v[k] = k < nb ? __ldca(xw + 32 * k) : 0.0f;
+            // block k's amax to lane k, which takes its scale
+            uint32_t m = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t mk = __reduce_max_sync(0xFFFFFFFFu, abs_bits(v[k]));
+                m = lane == k ? mk : m;
+            }
+            if (m >= kInfBits)
+                report_device_error(err, FP8_ERR_NONFINITE);
+            float s;
+            const uint32_t code = mx_block_scale<FMT>(m, s);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float sk = __shfl_sync(0xFFFFFFFFu, s, k);
+                if (k < nb)
+                    qw[32 * k] = enc1<FMT>(v[k], sk);
+            }
+            // (blocks past cols and padding rows: scale 1)
+            word = (lane < nb ? code : 127u) << (8 * (lane & 3));
+            word |= __shfl_xor_sync(0xFFFFFFFFu, word, 1);
+            word |= __shfl_xor_sync(0xFFFFFFFFu, word, 2);
+            word = __shfl_sync(0xFFFFFFFFu, word, lane >> 4 << 2);       // blocks 0 .. 3, 4 .. 7
         }
-        store_codes8<FMT>(q + r * ldq + c, in ? 8 : 0, qa, v, s);
-        // blocks past cols and padding rows: scale 1
-        uint32_t word = (in ? code : 127u) << (8 * ((lane >> 2) & 3));
-        word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
-        word |= __shfl_xor_sync(0xFFFFFFFFu, word, 8);
         const int64_t k = 2 * seg + (lane >> 4);              // k-block of this half warp
         if ((lane & 15) != 0 || k >= kb)
             continue;
@@ -1048,10 +1096,14 @@ int quantize_mx(const float* x, int64_t rows, int64_t cols, int64_t ldx, uint8_t
     const int64_t per_block = kThreads / 32;
     const int grid = static_cast<int>(std::min<int64_t>((windows + per_block - 1) / per_block, sm_count() * 16));
     int* err = device_error_word();
+    const auto launch = [&](auto* wide, auto* single) {
+        launch_dependent(xa >= 4 && qa >= 4 ? wide : single, grid, kThreads, st, x, rows, cols, ldx, xa, q, ldq, qa,
+                         scales, err);
+    };
     if (layout == 1)
-        launch_dependent(quant_mx_kernel<FMT, 1>, grid, kThreads, st, x, rows, cols, ldx, xa, q, ldq, qa, scales, err);
+        launch(quant_mx_kernel<FMT, 1, true>, quant_mx_kernel<FMT, 1, false>);
     else
-        launch_dependent(quant_mx_kernel<FMT, 0>, grid, kThreads, st, x, rows, cols, ldx, xa, q, ldq, qa, scales, err);
+        launch(quant_mx_kernel<FMT, 0, true>, quant_mx_kernel<FMT, 0, false>);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }

@@ -429,3 +429,29 @@ def test_mx_needs_no_workspace(gb, M):
 def test_mx_few_tiles_split_exact(gb, M, N, K, out):
     assert gb.gemm_fp8_mx_plan(M, N, K, out)["splits"] > 1
     _check_mx_exact(gb, M, N, K, out)
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(1, 32), (5, 288), (130, 512), (129, 4128)])
+def test_mx_quantize_mixed_alignments(gb, orc, layout, fmt, rows, cols):
+    """x and q of different alignment (either may rule the whole vectors
+    out); blocks of zeros, and a non-finite value reported from either form."""
+    x = _mx_inputs(rows, cols, seed=rows + cols)
+    x[rows - 1, :32] = 0.0
+    q_ref, s_ref = orc.mx_quantize(x, fmt)
+    want = s_ref if layout == 0 else tiled_layout(s_ref, rows, cols)
+    for pad, off, qpad, qoff in ((0, 0, 1, 0), (0, 4, 0, 3), (3, 0, 0, 0), (0, 8, 0, 4)):
+        xt = torch.zeros(rows * (cols + pad) + off, device="cuda")[off:].view(rows, cols + pad)[:, :cols]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((rows * (cols + qpad) + qoff,), 0xA5, dtype=torch.uint8, device="cuda")
+        qt = qb[qoff:].view(rows, cols + qpad)[:, :cols]
+        _, s = gb.fp8_quantize_mx(xt, fmt, scale_layout=layout, q=qt)
+        assert np.array_equal(qt.cpu().numpy(), q_ref)
+        assert np.array_equal(s.cpu().numpy(), want)
+        assert bool((qb[:qoff] == 0xA5).all())
+        assert bool((qb[qoff:].view(rows, cols + qpad)[:, cols:] == 0xA5).all())
+        assert gb.fp8_last_device_error() == 0
+        xt[rows // 2, cols - 1] = float("inf")
+        gb.fp8_quantize_mx(xt, fmt, scale_layout=layout, q=qt)
+        assert gb.fp8_last_device_error() == -4
