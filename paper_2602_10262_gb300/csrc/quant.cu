@@ -106,15 +106,16 @@ __device__ __forceinline__ void scale_from_amax(uint32_t amax_bits, float& s, fl
 // ---------------------------------------------------------------- rows in registers
 //
 // TPR threads (a warp, or a whole number of warps of one block) take a row,
-// each holding U vectors of W consecutive elements: vector u of thread t
-// starts at column (u * TPR + t) * W.  W = 8 is one 32-byte load a vector
-// (x 32-aligned, ldx % 8 == 0) or two 16-byte ones, with guarded scalar loads
-// past the last whole vector.  W = 1, where x or q allows neither, keeps a
-// warp's scalar loads and byte stores side by side: 4096 x 14336 at odd
-// offsets 49.9 us (four consecutive elements a thread 94.6, the row read twice
-// 86.2; 43.5 aligned).  Two 16-byte loads a vector, not vectors of four: half
-// as many addresses and guards, and the registers that they took left one
-// block an SM (the same size at 16-byte offsets 64.3 -> 45.6 us).
+// each holding U vectors of W = vector_of(A) consecutive elements: vector u of
+// thread t starts at column (u * TPR + t) * W.  A is the alignment of x's
+// rows in elements: 8, vectors of eight by one 32-byte load; 4, by two 16-byte
+// ones (guarded scalar loads past the last whole vector in both); 1, where x
+// or q allows neither, single elements, which keeps a warp's scalar loads and
+// byte stores side by side: 4096 x 14336 at odd offsets 49.9 us (four
+// consecutive elements a thread 94.6, the row read twice 86.2; 43.5 aligned).
+// Two 16-byte loads a vector, not vectors of four: half as many addresses and
+// guards, and the registers that they took left one block an SM (the same size
+// at 16-byte offsets 64.3 -> 45.6 us).
 //
 // What bounds it: HBM, once enough bytes are in flight.  Rows are loaded
 // once instead of twice (the second pass over L2 cost issue slots and load
@@ -179,20 +180,20 @@ __device__ __forceinline__ void load_8(const float* p, int64_t left, int xa, flo
         load_vec8(p, left, false, v);
 }
 
-// Max over the TPR threads of a row group.  red: one entry per warp of the
-// block, not in use by an earlier call since the last barrier.
-template <int TPR>
-__device__ __forceinline__ uint32_t row_max(uint32_t m, uint32_t* red)
+// Max over the tpr threads of a row group (tpr a power of two, the same for
+// the whole block).  red: one entry per warp of the block, not in use by an
+// earlier call since the last barrier; there is one barrier here if tpr > 32.
+__device__ __forceinline__ uint32_t row_max(uint32_t m, int tpr, uint32_t* red)
 {
     m = __reduce_max_sync(0xFFFFFFFFu, m);
-    if constexpr (TPR > 32) {
-        constexpr int kWarps = TPR / 32;
+    if (tpr > 32) {
+        const int warps = tpr / 32;
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         if (lane == 0)
             red[warp] = m;
         __syncthreads();
-        const int first = warp / kWarps * kWarps;
-        m = __reduce_max_sync(0xFFFFFFFFu, lane < kWarps ? red[first + lane] : 0u);
+        const int first = warp & ~(warps - 1);
+        m = __reduce_max_sync(0xFFFFFFFFu, lane < warps ? red[first + lane] : 0u);
     }
     return m;
 }
@@ -242,24 +243,29 @@ __device__ __forceinline__ uint8_t enc1(float v, float s)
     return static_cast<uint8_t>(enc2<FMT>(__fmul_rn(v, s), 0.0f) & 0xFFu);
 }
 
-// One row by its TPR threads (t: index within them; ok: the row exists).
-// xa, qa: alignment of the rows of x and q in elements (8, 4 or 1).
-template <int FMT, int TPR, int U, int W>
-__device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols, uint8_t* qr, float* d_out, int xa,
-                                                  int qa, int* err, uint32_t* red, int t, bool ok)
+__host__ __device__ constexpr int vector_of(int a)
 {
-    static_assert(W == 8 || W == 1, "whole vectors or single elements");
+    return a == 1 ? 1 : 8;
+}
+
+// One row by its tpr threads (t: index within them; ok: the row exists).
+// A, qa: alignment of the rows of x and q in elements (8, 4 or 1).
+template <int FMT, int U, int A>
+__device__ __forceinline__ void quantize_held_row(const float* xr, int cols, uint8_t* qr, float* d_out, int qa,
+                                                  int* err, int tpr, uint32_t* red, int t, bool ok)
+{
+    constexpr int W = vector_of(A);
     float v[U][W];
-    const int64_t n = ok ? cols : 0;
+    const int n = ok ? cols : 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+        const int c = (u * tpr + t) * W;
         if constexpr (W == 8)
-            load_8(xr + c, n - c, xa, v[u]);
+            load_8(xr + c, n - c, A, v[u]);
         else
             v[u][0] = c < n ? __ldca(xr + c) : 0.0f;
     }
-    const uint32_t m = row_max<TPR>(held_amax(v), red);
+    const uint32_t m = row_max(held_amax(v), tpr, red);
     float s, dq;
     scale_from_amax<FMT>(m, s, dq);
     if (t == 0 && ok) {
@@ -269,7 +275,7 @@ __device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols,
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+        const int c = (u * tpr + t) * W;
         if constexpr (W == 8)
             store_codes8<FMT>(qr + c, n - c, qa, v[u], s);
         else if (c < n)
@@ -277,12 +283,12 @@ __device__ __forceinline__ void quantize_held_row(const float* xr, int64_t cols,
     }
 }
 
-template <int FMT, int TPR, int U, int W>
+template <int FMT, int TPR, int U, int A>
 __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float* __restrict__ x, int64_t rows,
                                                                      int64_t cols, int64_t ldx,
                                                                      uint8_t* __restrict__ q, int64_t ldq,
-                                                                     float* __restrict__ d, int xa, int qa,
-                                                                     int early, int* err)
+                                                                     float* __restrict__ d, int qa, int early,
+                                                                     int* err)
 {
     grid_launch_dependents();
     __shared__ uint32_t red[2][32];
@@ -295,7 +301,7 @@ __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float
         if (r < rows) {
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int64_t c = static_cast<int64_t>(u * TPR + t) * W;
+                const int64_t c = static_cast<int64_t>(u * TPR + t) * vector_of(A);
                 if (c < cols)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(x + r * ldx + c));
             }
@@ -306,8 +312,7 @@ __global__ void __launch_bounds__(row_block<TPR>()) quant_row_kernel(const float
     for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRows; r0 < rows;
          r0 += static_cast<int64_t>(gridDim.x) * kRows, flip ^= 1) {
         const int64_t r = r0 + threadIdx.x / TPR;
-        quantize_held_row<FMT, TPR, U, W>(x + r * ldx, cols, q + r * ldq, d + r, xa, qa, err, red[flip], t,
-                                          r < rows);
+        quantize_held_row<FMT, U, A>(x + r * ldx, static_cast<int>(cols), q + r * ldq, d + r, qa, err, TPR, red[flip], t, r < rows);
     }
 }
 
@@ -352,7 +357,7 @@ __global__ void __launch_bounds__(row_block<TPR>()) quant_row_prune_kernel(const
             else
                 load_two_vec4(xr + c, n - c, v[u]);
         }
-        const uint32_t m = row_max<TPR>(held_amax(v), red[flip]);
+        const uint32_t m = row_max(held_amax(v), TPR, red[flip]);
         grid_launch_dependents();
         float s, dq;
         scale_from_amax<0>(m, s, dq);
@@ -484,42 +489,64 @@ __global__ void __launch_bounds__(kThreads) quant_long_row_prune_kernel(const fl
 }
 
 // Many independent per-row quantisations in one launch: the job table is
-// passed by value; CTA b takes global row b (rows of job j follow those of
-// job j - 1), held in the registers of kGroupedTpr threads (U: enough for
-// the longest row), or read twice where a row is longer than that allows.
+// passed by value.  A block of TB threads takes one unit at a time: as many
+// consecutive rows of one job as it has groups of that job's tpr threads.
+// Units of job j follow those of job j - 1.
+// Few rows (no more than two per SM) take a block of 512 each, for their own
+// latency.  Of many, a row takes the fewest threads (a warp up to the block)
+// that hold it in U vectors of eight each, so a launch may mix short rows and
+// long ones, in blocks of 256 up to 8192 columns, so that several are resident
+// on an SM.
+// One block of 512 a row whatever its length took as long for rows of 64 as
+// of 4096 columns: 32 jobs of 1024 rows of 64 columns 163 -> 10.6 us (85 with
+// a block of 256 a row that read it twice), of 1024 columns 162 -> 26.0 (97),
+// of 4096 166 -> 96 (116); 32 x 256 rows of 64 and 14336 columns in turn 79.2
+// -> 45.2 (48.2).
 struct RowJobs {
     fp8_quant_job job[FP8_QUANT_GROUPED_MAX];
-    int64_t row_start[FP8_QUANT_GROUPED_MAX + 1];
+    int64_t start[FP8_QUANT_GROUPED_MAX + 1];     // first unit of each job (read twice: first row)
     int xa[FP8_QUANT_GROUPED_MAX];        // alignment of the rows of x and of the codes, in elements: 8, 4 or 1
     int qa[FP8_QUANT_GROUPED_MAX];
+    int shift[FP8_QUANT_GROUPED_MAX];     // log2 of the threads per row
     int n;
 };
 
-constexpr int kGroupedTpr = 512;
-
-__device__ __forceinline__ int job_of_row(const RowJobs& jobs, int64_t g)
+__device__ __forceinline__ int job_of(const RowJobs& jobs, int64_t g)
 {
-    int j = 0;
-    while (j + 1 < jobs.n && jobs.row_start[j + 1] <= g)
-        ++j;
-    return j;
+    int lo = 0, hi = jobs.n;                      // start[lo] <= g < start[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if (jobs.start[mid] <= g)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
 }
 
-template <int U, int W>
-__global__ void __launch_bounds__(kGroupedTpr) quant_rows_grouped_kernel(const __grid_constant__ RowJobs jobs,
-                                                                         int* err)
+template <int TB, int U, int A, bool FEW>
+__global__ void __launch_bounds__(TB, (!FEW && U * vector_of(A) == 16 ? 1536 : 1024) / TB)
+    quant_rows_grouped_kernel(const __grid_constant__ RowJobs jobs, int* err)
 {
     grid_launch_dependents();
     grid_dependency_wait();
     __shared__ uint32_t red[2][32];
-    const int64_t total = jobs.row_start[jobs.n];
+    const int64_t total = jobs.start[jobs.n];
     int flip = 0;
-    for (int64_t g = blockIdx.x; g < total; g += gridDim.x, flip ^= 1) {
-        const int j = job_of_row(jobs, g);
+    for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
+        const int j = job_of(jobs, g);
         const fp8_quant_job& J = jobs.job[j];
-        const int64_t r = g - jobs.row_start[j];
-        quantize_held_row<0, kGroupedTpr, U, W>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r,
-                                                jobs.xa[j], jobs.qa[j], err, red[flip], threadIdx.x, true);
+        constexpr int kShift = TB == 512 ? 9 : 8;
+        const int shift = FEW ? kShift : jobs.shift[j], tpr = 1 << shift;
+        const int t = FEW ? threadIdx.x : threadIdx.x & (tpr - 1);
+        const int64_t unit = g - jobs.start[j];
+        const int64_t r = FEW ? unit : (unit << (kShift - shift)) + (threadIdx.x >> shift);
+        const float* xr = J.x + r * J.ldx;
+        uint8_t* qr = J.q + r * J.ldq;
+        quantize_held_row<0, U, A>(xr, static_cast<int>(J.cols), qr, J.dequant_scale + r, jobs.qa[j], err, tpr,
+                                   red[flip], t, FEW || r < J.rows);
+        if (tpr > 32)                             // (the buffers alternate from barrier to barrier)
+            flip ^= 1;
     }
 }
 
@@ -528,11 +555,11 @@ __global__ void __launch_bounds__(kThreads) quant_long_rows_grouped_kernel(const
 {
     grid_launch_dependents();
     __shared__ uint32_t red[kThreads / 32];
-    const int64_t total = jobs.row_start[jobs.n];
+    const int64_t total = jobs.start[jobs.n];
     for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
-        const int j = job_of_row(jobs, g);
+        const int j = job_of(jobs, g);
         const fp8_quant_job& J = jobs.job[j];
-        const int64_t r = g - jobs.row_start[j];
+        const int64_t r = g - jobs.start[j];
         quantize_row<0>(J.x + r * J.ldx, J.cols, J.q + r * J.ldq, J.dequant_scale + r, jobs.xa[j] >= 4 && jobs.qa[j] >= 4,
                         err, red);
     }
@@ -574,7 +601,7 @@ __global__ void __launch_bounds__(kClusterThreads) quant_cluster_kernel(const fl
         c[u] = (i - r[u] * per_row) * 8;
         load_8(x + r[u] * ldx + c[u], r[u] < rows ? cols - c[u] : 0, xa, v[u]);
     }
-    uint32_t m = row_max<kClusterThreads>(held_amax(v), red);
+    uint32_t m = row_max(held_amax(v), kClusterThreads, red);
     if (threadIdx.x == 0)
         cta_max = m;
     cluster_sync();
@@ -794,12 +821,16 @@ struct RowLaunch {
     {
         const int xa = row_align(x, ldx, 4), qa = row_align(q, ldq, 1);
         const int grid = row_grid(rows, row_block<TPR>() / TPR);
-        if (xa >= 4 && qa >= 4)
-            launch_dependent(quant_row_kernel<FMT, TPR, U, 8>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q, ldq,
-                             d, xa, qa, rows <= 2 * sm_count(), err);
+        const auto launch = [&](auto* kernel) {
+            launch_dependent(kernel, grid, row_block<TPR>(), st, x, rows, cols, ldx, q, ldq, d, qa,
+                             rows <= 2 * sm_count(), err);
+        };
+        if (xa == 8 && qa >= 4)
+            launch(quant_row_kernel<FMT, TPR, U, 8>);
+        else if (xa == 4 && qa >= 4)
+            launch(quant_row_kernel<FMT, TPR, U, 4>);
         else
-            launch_dependent(quant_row_kernel<FMT, TPR, 8 * U, 1>, grid, row_block<TPR>(), st, x, rows, cols, ldx, q,
-                             ldq, d, xa, qa, rows <= 2 * sm_count(), err);
+            launch(quant_row_kernel<FMT, TPR, 8 * U, 1>);
     }
 };
 
@@ -1209,7 +1240,7 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
     RowJobs rj;
     memset(&rj, 0, sizeof(rj));
     int64_t rows = 0, max_cols = 0;
-    bool wide = true;
+    int a = 8;                                    // the least alignment of any job's rows
     for (int i = 0; i < num_jobs; ++i) {
         const fp8_quant_job& J = jobs[i];
         if (J.rows < 0 || J.cols < 0)
@@ -1225,35 +1256,58 @@ extern "C" int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job* jobs, int num
             return FP8_ERR_ALIGN;
         const int k = rj.n++;
         rj.job[k] = J;
-        rj.row_start[k] = rows;
         rj.xa[k] = row_align(J.x, J.ldx, 4);
         rj.qa[k] = row_align(J.q, J.ldq, 1);
-        wide = wide && rj.xa[k] >= 4 && rj.qa[k] >= 4;
+        a = std::min(a, rj.qa[k] >= 4 ? rj.xa[k] : 1);
         max_cols = std::max(max_cols, J.cols);
         rows += J.rows;
     }
-    rj.row_start[rj.n] = rows;
     if (rows == 0)
         return FP8_OK;
     if (!device_supported())
         return FP8_ERR_UNSUPPORTED;
-    const int grid = row_grid(rows, 1);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     int* err = device_error_word();
-    const auto launch = [&](auto* w8, auto* w1) {
-        if (wide)
-            launch_dependent(w8, grid, kGroupedTpr, st, rj, err);
-        else
-            launch_dependent(w1, grid, kGroupedTpr, st, rj, err);
+    // threads a block and vectors a thread (see quant_rows_grouped_kernel)
+    const bool few = rows <= 2 * sm_count();
+    const bool held = max_cols <= 4 * 8 * 512;
+    const int tb = few || max_cols > 4 * 8 * 256 ? 512 : 256;
+    const int u = max_cols > 2 * 8 * tb ? 4 : (few && max_cols <= 8 * tb ? 1 : 2);
+    int64_t units = 0;
+    for (int i = 0; i < rj.n; ++i) {
+        int shift = few ? 9 : 5;
+        while ((1 << shift) < tb && (int64_t{8} * u << shift) < rj.job[i].cols)
+            ++shift;
+        const int per_unit = held ? tb >> shift : 1;
+        rj.shift[i] = shift;
+        rj.start[i] = units;
+        units += (rj.job[i].rows + per_unit - 1) / per_unit;
+    }
+    rj.start[rj.n] = units;
+    const int grid = row_grid(units, 1);
+    const auto launch = [&](auto* a8, auto* a4, auto* a1) {
+        launch_dependent(a == 8 ? a8 : a == 4 ? a4 : a1, grid, tb, st, rj, err);
     };
-    if (max_cols <= 8 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<1, 8>, quant_rows_grouped_kernel<8, 1>);
-    else if (max_cols <= 16 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<2, 8>, quant_rows_grouped_kernel<16, 1>);
-    else if (max_cols <= 32 * kGroupedTpr)
-        launch(quant_rows_grouped_kernel<4, 8>, quant_rows_grouped_kernel<32, 1>);
-    else
+    if (!held)
         quant_long_rows_grouped_kernel<<<grid, kThreads, 0, st>>>(rj, err);
+    else if (few && u == 1)
+        launch(quant_rows_grouped_kernel<512, 1, 8, true>, quant_rows_grouped_kernel<512, 1, 4, true>,
+               quant_rows_grouped_kernel<512, 8, 1, true>);
+    else if (few && u == 2)
+        launch(quant_rows_grouped_kernel<512, 2, 8, true>, quant_rows_grouped_kernel<512, 2, 4, true>,
+               quant_rows_grouped_kernel<512, 16, 1, true>);
+    else if (few)
+        launch(quant_rows_grouped_kernel<512, 4, 8, true>, quant_rows_grouped_kernel<512, 4, 4, true>,
+               quant_rows_grouped_kernel<512, 32, 1, true>);
+    else if (u == 2)
+        launch(quant_rows_grouped_kernel<256, 2, 8, false>, quant_rows_grouped_kernel<256, 2, 4, false>,
+               quant_rows_grouped_kernel<256, 16, 1, false>);
+    else if (tb == 256)
+        launch(quant_rows_grouped_kernel<256, 4, 8, false>, quant_rows_grouped_kernel<256, 4, 4, false>,
+               quant_rows_grouped_kernel<256, 32, 1, false>);
+    else
+        launch(quant_rows_grouped_kernel<512, 4, 8, false>, quant_rows_grouped_kernel<512, 4, 4, false>,
+               quant_rows_grouped_kernel<512, 32, 1, false>);
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;
 }

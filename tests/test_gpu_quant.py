@@ -348,3 +348,33 @@ def test_row_mixed_alignments(gb, orc, rows, cols):
         assert gb.library().fp8_quantize_e4m3_rows_grouped(job, 1, torch.cuda.current_stream().cuda_stream) == 0
         assert torch.equal(qb, single) and np.array_equal(d.cpu().numpy(), do)
     assert gb.fp8_last_device_error() == 0
+
+
+@pytest.mark.parametrize("rows", [1, 15, 17, 130])
+@pytest.mark.parametrize("lengths", [(1,), (256, 257), (512, 513, 100), (4096, 40, 4097), (8192, 3, 513),
+                                     (16384, 64, 8193, 256, 1024, 2049), (16385, 64)])
+def test_grouped_units_of_mixed_lengths(gb, orc, rows, lengths):
+    """Rows of every threads-per-row shape in one launch (a block takes as
+    many short rows as it has warps), row counts that end inside a block,
+    aligned and unaligned jobs side by side; nothing written between rows."""
+    from paper_2602_10262_gb300._lib import FP8QuantJob
+    mats, jobs = [], []
+    for i, c in enumerate(lengths * 2):
+        n = rows + i
+        x = workloads.randn_f32((n, c), seed=100 * i + c)
+        x[n - 1, c - 1] = 500.0
+        pad = -c % 8 if i < len(lengths) else 1
+        xt = torch.zeros((n, c + pad), device="cuda")[:, :c]
+        xt.copy_(torch.from_numpy(x))
+        qb = torch.full((n, c + pad), 0xA5, dtype=torch.uint8, device="cuda")
+        d = torch.empty(n, device="cuda")
+        mats.append((x, xt, qb, d, c))
+        jobs.append(FP8QuantJob(xt.data_ptr(), n, c, xt.stride(0), qb.data_ptr(), qb.stride(0), d.data_ptr()))
+    arr = (FP8QuantJob * len(jobs))(*jobs)
+    for _ in range(2):
+        assert gb.library().fp8_quantize_e4m3_rows_grouped(arr, len(arr), torch.cuda.current_stream().cuda_stream) == 0
+    for x, _, qb, d, c in mats:
+        qo, do = orc.quantize(x, 1)
+        assert np.array_equal(qb[:, :c].cpu().numpy(), qo) and np.array_equal(d.cpu().numpy(), do)
+        assert bool((qb[:, c:] == 0xA5).all())
+    assert gb.fp8_last_device_error() == 0
