@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(kThreads) decompress24_vec_kernel(const uint2*
     }
 }
 
-// The inverse for any K % 4 == 0 and any alignment, by the same pieces.
+// The inverse for any K % 4 == 0 and any alignment of its inputs, out on a
+// 4-byte boundary, by the same pieces.
 template <int U>
 __global__ void __launch_bounds__(kThreads) decompress24_any_kernel(const uint8_t* __restrict__ vals, int v_align,
                                                                     const uint8_t* __restrict__ meta, int m_align,
@@ -292,6 +293,56 @@ __global__ void __launch_bounds__(kThreads) decompress24_any_kernel(const uint8_
     }
 }
 
+// The inverse with out off a 4-byte boundary: one group a thread and step, as
+// the 16 single bytes that a thread of the kernel above would store one by one,
+// 16 apart from its neighbour's, write every sector 16 times (16384 x 4100 from
+// an odd byte: 180 us, 51.6 this way; 16384 x 14336 586 and 156).  Kept codes and output have no gaps
+// between rows, so a group's place in them is its index alone; ROWS: metadata
+// rows end in half a byte, and only they need the row (a thread's next group
+// is step_rows rows and step_groups groups on: one division a thread).
+template <int U, bool ROWS>
+__global__ void __launch_bounds__(kThreads) decompress24_group_kernel(const uint8_t* __restrict__ vals, int v_align,
+                                                                      const uint8_t* __restrict__ meta, PieceShape s,
+                                                                      int step_rows, int step_groups,
+                                                                      uint8_t* __restrict__ out, int o_align)
+{
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads * U);
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kThreads * U) + threadIdx.x; i0 < s.total; i0 += step) {
+        uint32_t v[U][1], m[U];
+        int64_t r = 0, p = i0;
+        if (ROWS)
+            piece_row(s, i0, &r, &p);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * kThreads;
+            if (ROWS && u > 0) {
+                r += step_rows;
+                p += step_groups;
+                if (p >= s.per_row) {
+                    p -= s.per_row;
+                    ++r;
+                }
+            } else if (!ROWS) {
+                p = i;
+            }
+            if (i < s.total) {
+                load_words<1>(vals + 2 * i, 2, v_align, v[u]);
+                m[u] = __ldca(meta + r * s.ldm + (p >> 1)) >> (4 * (p & 1));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * kThreads;
+            if (i < s.total) {
+                const uint32_t w[1] = {expand_group(v[u][0], m[u])};
+                store_words<1>(out + 4 * i, 4, o_align, w);
+            }
+        }
+    }
+}
+
 // The largest of 16, 8, 4, 2, 1 that divides a base address and a row stride.
 int bytes_align(const void* p, int64_t ld)
 {
@@ -299,9 +350,9 @@ int bytes_align(const void* p, int64_t ld)
     return static_cast<int>(v & (~v + 1));
 }
 
-PieceShape piece_shape(int64_t M, int64_t K)
+PieceShape piece_shape(int64_t M, int64_t K, int groups = 4)
 {
-    const int64_t per_row = (K + 15) / 16;
+    const int64_t per_row = (K + 4 * groups - 1) / (4 * groups);
     return {M * per_row, per_row, K / 4, K / 2, (K + 7) / 8};
 }
 
@@ -396,12 +447,22 @@ extern "C" int prune24_decompress(const uint8_t* a_vals, const uint8_t* a_meta, 
             launch_dependent(decompress24_vec_kernel<kPieces>, static_cast<unsigned>(blocks), kThreads, st, v8, m2,
                              pieces, o16);
     } else {
-        const PieceShape s = piece_shape(M, K);
-        const int u = pieces_per_thread(s.total);
-        const int va = bytes_align(a_vals, M == 1 ? 0 : s.ldv), ma = bytes_align(a_meta, M == 1 ? 0 : s.ldm),
-                  oa = bytes_align(out, M == 1 ? 0 : K);
-        launch_dependent(u == 1 ? decompress24_any_kernel<1> : decompress24_any_kernel<kPieces>,
-                         piece_grid(s.total, u), kThreads, st, a_vals, va, a_meta, ma, s, out, K, oa);
+        const int oa = bytes_align(out, M == 1 ? 0 : K);
+        const PieceShape s = piece_shape(M, K, oa < 4 ? 1 : 4);
+        const int u = pieces_per_thread(oa < 4 ? s.total / 2 : s.total);
+        const int va = bytes_align(a_vals, M == 1 ? 0 : s.ldv), ma = bytes_align(a_meta, M == 1 ? 0 : s.ldm);
+        if (oa < 4) {
+            const bool rows = K % 8 != 0 && M > 1;
+            launch_dependent(rows ? (u == 1 ? decompress24_group_kernel<1, true>
+                                            : decompress24_group_kernel<kPieces, true>)
+                                  : (u == 1 ? decompress24_group_kernel<1, false>
+                                            : decompress24_group_kernel<kPieces, false>),
+                             piece_grid(s.total, u), kThreads, st, a_vals, va, a_meta, s,
+                             static_cast<int>(kThreads / s.per_row), static_cast<int>(kThreads % s.per_row), out, oa);
+        } else {
+            launch_dependent(u == 1 ? decompress24_any_kernel<1> : decompress24_any_kernel<kPieces>,
+                             piece_grid(s.total, u), kThreads, st, a_vals, va, a_meta, ma, s, out, K, oa);
+        }
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;

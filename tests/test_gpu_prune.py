@@ -100,3 +100,23 @@ def test_expand_any_index_nibble(orc):
     off = buf[4:].reshape(M, K)
     gb.prune24_decompress(vals, meta, K, out=off)
     assert torch.equal(off, out)
+
+
+@pytest.mark.parametrize("M,K", [(1, 4), (1, 8), (3, 12), (7, 20), (5, 132), (33, 28), (320, 4100), (129, 1032),
+                                 (9, 4096), (1300, 4100), (40000, 4), (20000, 12), (700, 8200)])
+def test_expand_to_any_byte(orc, M, K):
+    """Outputs that start off a 4-byte boundary (one group a thread, with few
+    groups and many, rows of whole and of half metadata bytes) equal the
+    oracle; nothing is written beside them."""
+    import paper_2602_10262_gb300 as gb
+    vo, mo = orc.prune24(workloads.random_codes((M, K), seed=9 + M + K))
+    want = orc.decompress24(vo, mo, K)
+    for shift, off in ((0, 1), (0, 2), (1, 3), (2, 7)):
+        vb = torch.zeros(M * (K // 2) + shift, dtype=torch.uint8, device="cuda")
+        v, m = vb[shift:].view(M, -1), torch.from_numpy(mo).cuda()
+        v.copy_(torch.from_numpy(vo))
+        buf = torch.full((M * K + off + 5,), 0xA5, dtype=torch.uint8, device="cuda")
+        out = buf[off:-5].view(M, K)
+        gb.prune24_decompress(v, m, K, out=out)
+        assert np.array_equal(out.cpu().numpy(), want)
+        assert bool((buf[:off] == 0xA5).all()) and bool((buf[-5:] == 0xA5).all())
