@@ -73,10 +73,10 @@ __global__ void __launch_bounds__(kThreads) prune24_vec_kernel(const uint8_t* __
     }
 }
 
-// Any K % 4 == 0 and any alignment: a row is ceil(K / 16) pieces of up to
-// four groups, and a thread takes U pieces of the whole matrix (kThreads
-// apart, the row by one 32-bit division), each with the widest loads and
-// stores its arrays allow.  16384 x 4100 (rows of half metadata bytes): 28.6
+// Any K % 4 == 0 and any alignment: a row is pieces of up to four groups (G),
+// and a thread takes U pieces of the whole matrix (kThreads apart, the row by
+// one 32-bit division), each with the widest loads and stores its arrays
+// allow.  16384 x 4100 (rows of half metadata bytes): 28.6
 // us, and 46.2 to expand it again; one metadata byte, or one group, per
 // thread with single-byte accesses and a 64-bit division took 46.8 and 54.9.
 struct PieceShape {
@@ -163,7 +163,12 @@ __device__ __forceinline__ void store_words(uint8_t* p, int n, int align, const 
     }
 }
 
-template <int U>
+// Pieces of two groups (G = 2) where a or the kept codes start on any byte and
+// there is too little work to fill the SMs: sixteen single-byte loads, or eight
+// stores, one after the other are then all the time there is (320 x 4100: 3.7
+// us with four groups a thread, 2.6 with two).  Not for short rows of half
+// metadata bytes, which lose more to their last piece (4096 x 132: 1.9, 2.2).
+template <int U, int G>
 __global__ void __launch_bounds__(kThreads) prune24_any_kernel(const uint8_t* __restrict__ a, PieceShape s,
                                                                int64_t lda, int a_align, uint8_t* __restrict__ vals,
                                                                int v_align, uint8_t* __restrict__ meta, int m_align)
@@ -172,7 +177,7 @@ __global__ void __launch_bounds__(kThreads) prune24_any_kernel(const uint8_t* __
     grid_dependency_wait();
     const int64_t step = static_cast<int64_t>(gridDim.x) * (kThreads * U);
     for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kThreads * U) + threadIdx.x; i0 < s.total; i0 += step) {
-        uint32_t w[U][4];
+        uint32_t w[U][G];
         int64_t r[U], p[U];
         int n[U];                          // groups of the piece
 #pragma unroll
@@ -181,19 +186,23 @@ __global__ void __launch_bounds__(kThreads) prune24_any_kernel(const uint8_t* __
             n[u] = 0;
             if (i < s.total) {
                 piece_row(s, i, &r[u], &p[u]);
-                n[u] = static_cast<int>(min(static_cast<int64_t>(4), s.groups - 4 * p[u]));
-                load_words<4>(a + r[u] * lda + 16 * p[u], 4 * n[u], a_align, w[u]);
+                n[u] = static_cast<int>(min(static_cast<int64_t>(G), s.groups - G * p[u]));
+                load_words<G>(a + r[u] * lda + 4 * G * p[u], 4 * n[u], a_align, w[u]);
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (n[u] == 0)
                 continue;
-            uint32_t v[2];
-            const uint32_t nib =
-                select_groups4(w[u][0], w[u][1], w[u][2], w[u][3], &v[0], &v[1]) & ((1u << (4 * n[u])) - 1u);
-            store_words<2>(vals + r[u] * s.ldv + 8 * p[u], 2 * n[u], v_align, v);
-            uint8_t* md = meta + r[u] * s.ldm + 2 * p[u];
+            uint32_t v01, v23;
+            const uint32_t nib = select_groups4(w[u][0], w[u][1], G == 4 ? w[u][G - 2] : 0u, G == 4 ? w[u][G - 1] : 0u,
+                                                &v01, &v23) & ((1u << (4 * n[u])) - 1u);
+            uint32_t v[G / 2];
+            v[0] = v01;
+            if constexpr (G == 4)
+                v[1] = v23;
+            store_words<G / 2>(vals + r[u] * s.ldv + 2 * G * p[u], 2 * n[u], v_align, v);
+            uint8_t* md = meta + r[u] * s.ldm + G / 2 * p[u];
             if (m_align >= 2 && n[u] > 2) {
                 *reinterpret_cast<uint16_t*>(md) = static_cast<uint16_t>(nib);
             } else {
@@ -402,12 +411,17 @@ extern "C" int prune24_compress(const uint8_t* a, int64_t M, int64_t K, int64_t 
         else
             launch_dependent(prune24_vec_kernel<kPieces>, dim3(gx, gy), kThreads, st, a, M, K, lda, a_vals, a_meta);
     } else {
-        const PieceShape s = piece_shape(M, K);
+        PieceShape s = piece_shape(M, K);
         const int u = pieces_per_thread(s.total);
         const int aa = bytes_align(a, row_a), va = bytes_align(a_vals, M == 1 ? 0 : s.ldv),
                   ma = bytes_align(a_meta, M == 1 ? 0 : s.ldm);
-        launch_dependent(u == 1 ? prune24_any_kernel<1> : prune24_any_kernel<kPieces>, piece_grid(s.total, u),
-                         kThreads, st, a, s, lda, aa, a_vals, va, a_meta, ma);
+        const bool halves = u == 1 && std::min(aa, va) == 1 && (K % 8 == 0 || K >= 1024);
+        if (halves)
+            s = piece_shape(M, K, 2);
+        launch_dependent(halves    ? prune24_any_kernel<1, 2>
+                         : u == 1 ? prune24_any_kernel<1, 4>
+                                  : prune24_any_kernel<kPieces, 4>,
+                         piece_grid(s.total, u), kThreads, st, a, s, lda, aa, a_vals, va, a_meta, ma);
     }
     GB_CUDA_OK(cudaGetLastError());
     return FP8_OK;

@@ -102,6 +102,28 @@ def test_expand_any_index_nibble(orc):
     assert torch.equal(off, out)
 
 
+@pytest.mark.parametrize("M,K", [(1, 4), (1, 8), (3, 12), (7, 20), (5, 132), (320, 4100), (129, 1032), (9, 4096),
+                                 (1300, 4100)])
+@pytest.mark.parametrize("pad,off", [(0, 1), (1, 0), (5, 3)])
+def test_compress_from_any_byte(orc, M, K, pad, off):
+    """Codes that start on any byte: two groups a thread while there is little
+    work (the last shape is past that), outputs aligned and not, nothing
+    written beside them."""
+    import paper_2602_10262_gb300 as gb
+    a = workloads.random_codes((M, K), seed=5 + M + K)
+    t = torch.zeros(M * (K + pad) + off, dtype=torch.uint8, device="cuda")[off:].view(M, K + pad)[:, :K]
+    t.copy_(torch.from_numpy(a))
+    vo, mo = orc.prune24(a)
+    for shift in (0, 1, 2):
+        vb = torch.full((M * (K // 2) + shift + 4,), 0xA5, dtype=torch.uint8, device="cuda")
+        mb = torch.full((M * ((K + 7) // 8) + shift + 4,), 0xA5, dtype=torch.uint8, device="cuda")
+        v, m = vb[shift:-4].view(M, -1), mb[shift:-4].view(M, -1)
+        gb.prune24_compress(t, v, m)
+        assert np.array_equal(v.cpu().numpy(), vo) and np.array_equal(m.cpu().numpy(), mo)
+        for b in (vb, mb):
+            assert bool((b[:shift] == 0xA5).all()) and bool((b[-4:] == 0xA5).all())
+
+
 @pytest.mark.parametrize("M,K", [(1, 4), (1, 8), (3, 12), (7, 20), (5, 132), (33, 28), (320, 4100), (129, 1032),
                                  (9, 4096), (1300, 4100), (40000, 4), (20000, 12), (700, 8200)])
 def test_expand_to_any_byte(orc, M, K):
