@@ -2266,28 +2266,43 @@ TileChoice choose(const Job* jobs, const int* bns, int n, int max_ctas, const Ti
 // cycles, fitted to a sweep of widths 112..256 over nine products (512 to
 // 4096 rows, K 4096 to 14336): it falls with the width far less than the
 // MMAs do, the loads of A and their latency being the rest.  Results do not
-// depend on the width: a column's sum is its own.  Measured against full
-// width, L2-cold: 512 x 12288 x 4096 27.0 -> 24.9 us (176 wide: two full
-// waves instead of one and a quarter), 2048 x 5120 x 4096 35.5 -> 34.1, 2:4
-// 512 x 14336 x 4096 33.1 -> 28.3; a wave more than needed loses as much
-// (4096^3: 45.5 us at 224, 51.1 at 208), and a narrower tile in the same one
-// wave gains nothing (512 x 8192 x 8192 at 224).
+// depend on the width: a column's sum is its own.
+// Where the k-loop is short the last wave's few tiles run faster than those of
+// a full one, and the fit promises more than there is; there full width stays.
+// Measured against full width in one process, L2-cold, bf16 out (a summary over
+// 769 products is in profiles/gemm_fp8_kernel_pair_width.json): dense, K 1024
+// 1 to 5 % slower, 1536 level, from 2048 on 2, from 4096 on 5, 14336 8 %
+// faster (medians; 512 x 10240 x 4096 26.5 -> 24.0 us).  2:4 has half the bytes
+// of A and gains less: up to K 2048 as much as 11 % slower, 3072 and 4096 level
+// and 1 to 7 % faster for 192 (1000 x 5120 x 4096 20.9 -> 19.7; transposed
+// outputs 5 % slower to 5 % faster, so not there), from 6144 on 2 %; faster at
+// every K where the width leaves out a tenth of the columns, padding (8192 x
+// 512 x 1024: 10.7 -> 9.9 us), or where unaligned output rows make the epilogue
+// the longest part of a tile (1536 x 3001 x 1024: 22.0 -> 15.6).
 int pair_width(const Job& j, int widest, int pairs)
 {
     const bool sparse = j.E != nullptr;
     const int64_t m_blocks = (j.rows_p + 2 * BM - 1) / (2 * BM);
-    const double k_blocks = static_cast<double>((j.K + BK - 1) / BK);
+    const int64_t k_blocks = (j.K + BK - 1) / BK;
+    const bool unaligned = !aligned16(j.C) || j.ldc * (j.out_bf16 ? 2 : 4) % 16 != 0;
     constexpr double kLaunch = 12400;             // cycles of a launch beside its tiles (6 us)
+    const auto columns = [&](int w) { return (j.rows_q + w - 1) / w * w; };
     const auto cost = [&](int w) {
-        const int64_t tiles = m_blocks * ((j.rows_q + w - 1) / w);
+        const int64_t tiles = m_blocks * (columns(w) / w);
         const int64_t waves = (tiles + pairs - 1) / pairs;
         const double block = sparse ? 318 + 1.26 * w : 462 + 0.78 * w;
-        return kLaunch + static_cast<double>(waves) * k_blocks * block;
+        return kLaunch + static_cast<double>(waves * k_blocks) * block;
+    };
+    const auto measured_faster = [&](int w) {
+        if (!sparse)
+            return k_blocks >= 16;
+        return k_blocks >= 48 || (k_blocks >= 24 && w >= 192 && !j.trans_out) || unaligned ||
+               10 * columns(w) <= 9 * columns(widest);
     };
     int best = widest;
     double best_cost = 0.95 * cost(widest);
     for (int w = widest - 16; w >= 128; w -= 16) {
-        if (cost(w) < best_cost) {
+        if (measured_faster(w) && cost(w) < best_cost) {
             best = w;
             best_cost = cost(w);
         }

@@ -247,3 +247,17 @@ def test_narrow_pair_tiles_are_planned(gb):
     assert gb.gemm_fp8_dense_plan(16384, 16384, 16384)["bn"] == 256
     assert gb.gemm_fp8_sparse24_plan(14336, 512, 4096)["bn"] < 224
     assert gb.gemm_fp8_sparse24_plan(16384, 16384, 16384)["bn"] == 224
+
+
+def test_short_k_loops_keep_full_width(gb):
+    """Short products take narrow pair tiles only where those were measured
+    faster: less padding, or unaligned output rows."""
+    for M, N, K in ((1000, 5120, 1024), (700, 7168, 1024), (6144, 1024, 1536)):
+        p = gb.gemm_fp8_dense_plan(M, N, K)
+        assert p["mt"] == 3 and p["bn"] == 256, (M, N, K, p)
+    for M, N, K in ((4096, 2048, 1024), (1024, 5120, 1024), (384, 10240, 2048), (6144, 1024, 2048)):
+        p = gb.gemm_fp8_sparse24_plan(M, N, K)
+        assert p["mt"] == 3 and p["bn"] == 224, (M, N, K, p)
+    for M, N, K in ((8192, 512, 1024), (14336, 256, 2048), (1536, 3001, 1024)):
+        p = gb.gemm_fp8_sparse24_plan(M, N, K)
+        assert p["mt"] == 3 and p["bn"] < 224, (M, N, K, p)
