@@ -1496,27 +1496,18 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                     tmem_ld_32x32b_x16(taddr + c_lo + 16 * h, held[h]);
                 tmem_ld_wait();
                 release();
-                if (!P.trans_out) {
-                    if (P.out_bf16)
-                        epilogue_rows_coalesced<2, LB, C::kEpiBufs, C::kDrainFirst>(
-                            P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo, c_hi, held);
-                    else
-                        epilogue_rows_coalesced<4, LB, C::kEpiBufs, C::kDrainFirst>(
-                            P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo, c_hi, held);
-                } else {
-                    float s_cur = 0.0f;
-#pragma unroll
-                    for (int h = 0; h < C::kDrainFirst / 16; ++h) {
-                        if (h % 2 == 0)
-                            s_cur = sw.take(P, jbase + c_lo, lane);
-                        store_chunk16(P, i, row_ok, fi, jbase + c_lo + 16 * h, held[h], s_cur, 16 * (h & 1));
-                    }
-                }
+                if (P.out_bf16)
+                    epilogue_rows_coalesced<2, LB, C::kEpiBufs, C::kDrainFirst>(P, taddr, row0, fi, jbase, buf, lane,
+                                                                                sw, tmC, c_lo, c_hi, held);
+                else
+                    epilogue_rows_coalesced<4, LB, C::kEpiBufs, C::kDrainFirst>(P, taddr, row0, fi, jbase, buf, lane,
+                                                                                sw, tmC, c_lo, c_hi, held);
                 c_lo = acc ? C::kDrainFirst : 0;
                 c_hi = acc ? c_end : c_end - C::kDrainFirst;
                 sw.init(P, jbase + c_lo, lane, c_hi - c_lo);
             }
-            if (!P.trans_out) {
+            // (block-scaled pairs are never transposed: build_plan_tiles)
+            if (!P.trans_out || (PAIR && MX)) {
                 if (P.out_bf16)
                     epilogue_rows_coalesced<2, LB, C::kEpiBufs>(P, taddr, row0, fi, jbase, buf, lane, sw, tmC, c_lo,
                                                                c_hi);
@@ -2318,8 +2309,8 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
     const TileChoice c = choose(jobs, bns_in, n, max_ctas, expl);
     const bool sparse = n > 0 && jobs[0].E != nullptr;     // all alike when mt == 2
     // N tile widths: the problems' own, under the tuned cap if any (block-
-    // scaled launches: 128 or 256, as gemm_fp8_mx chose)
-    int bns[MAXP > 0 ? MAXP : 1];
+    // scaled launches: as gemm_fp8_mx chose)
+    int bns[MAXP > 0 ? MAXP : 1] = {};
     for (int i = 0; i < n; ++i)
         bns[i] = (c.bn_cap > 0 && jobs[i].sfp == nullptr) ? std::min(bns_in[i], c.bn_cap) : bns_in[i];
     int max_bn = 0;
@@ -2347,11 +2338,15 @@ int build_plan_tiles(Params<MAXP>& prm, const Job* jobs, const int* bns_in, int 
     prm.group_m = c.group_m;
     if (n > 0 && jobs[0].sfp != nullptr) {
         // block-scaled launches (single problems): CTA pairs or 128 x 256
-        // tiles (one accumulator, the scale ring after it) or 128 x 128
-        // tiles (two)
+        // tiles (one accumulator, the scale ring after it), or 128-row tiles
+        // up to 128 wide (two)
         if constexpr (MAXP == 1) {
             // pairs: two accumulators with shared columns once a pair takes a
-            // second tile (see the MX comment at Cfg)
+            // second tile (see the MX comment at Cfg); their epilogues store
+            // rows only (a transposed product has at most 128 columns, which
+            // no pair takes)
+            if (c.mt == 3 && jobs[0].trans_out)
+                return FP8_ERR_UNSUPPORTED;
             if (c.mt == 3)
                 return 2 * prm.prob[0].m_blocks * prm.prob[0].n_blocks > (max_ctas > 0 ? max_ctas : sm_count())
                            ? plan<MAXP, 1, false, BN_MAX, 2, 2, true>(prm, max_ctas, pl)
