@@ -288,19 +288,38 @@ __device__ __forceinline__ void abort_pipeline(volatile int* flag, int* err)
 // add their latency to the epilogue.  Ordinary loads, not the read-only path:
 // that one is for data nothing writes while the kernel runs, and the kernel
 // before this one, often the quantiser of these very scales, may still be
-// running when this grid starts.
+// running when this grid starts.  Plain ones mostly: the load intrinsics are
+// volatile assembly, which holds the code around them in place and took 0.1 to
+// 0.2 us of every tile wider than 16 columns with four epilogue warps (128 x
+// 14336 x 256 5.62 -> 5.82 us, plain 5.62) and up to 5 % of 2:4 pairs.  Dense
+// kernels with eight are better off with the intrinsic (PINNED; 4096 x 4096 x
+// 256 15.76 us, plain 15.96).
+template <bool PINNED>
+__device__ __forceinline__ float load_scale(const float* p)
+{
+    if constexpr (PINNED)
+        return __ldca(p);
+    else
+        return *p;
+}
+
 struct ScaleWindows {
     float w0, w1;           // the next two windows to hand out
     int next;               // column (from the first) of the window after w1
     int width;              // columns this warp covers
+    bool pinned;            // constant per kernel (load_scale)
 
-    __device__ __forceinline__ static float load(const ProblemScalars& P, int j, int lane)
+    __device__ __forceinline__ float load(const ProblemScalars& P, int j, int lane) const
     {
         j += lane;
-        return j < P.rows_q ? __ldca(P.sq + (P.sq_mode ? j : 0)) : 0.0f;
+        if (j >= P.rows_q)
+            return 0.0f;
+        const float* s = P.sq + (P.sq_mode ? j : 0);
+        return pinned ? load_scale<true>(s) : load_scale<false>(s);
     }
-    __device__ __forceinline__ void init(const ProblemScalars& P, int jbase, int lane, int cols)
+    __device__ __forceinline__ void init(const ProblemScalars& P, int jbase, int lane, int cols, bool pin)
     {
+        pinned = pin;
         width = cols;
         w0 = load(P, jbase, lane);
         w1 = cols > 32 ? load(P, jbase + 32, lane) : 0.0f;
@@ -1326,6 +1345,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
         // warp w reads TMEM lanes 32 (w % 4) ..; with 256-row tiles of half
         // (w - 2) / 4, with two warps per lane quarter of columns [0, mid) or
         // [mid, bn) (mid: half the tile rounded up to 64 columns)
+        constexpr bool kPinScales = C::kEpiWarps == 8 && !SP;
         const int quarter = warp & 3;
         const int half = MT == 2 ? (warp - 2) >> 2 : 0;
         const int cpart = C::kEpiSplit == 2 ? (warp - 2) >> 2 : 0;
@@ -1342,7 +1362,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
             // (pairs: CTA r holds rows 128 r .. of the 256-row tile)
             const int i = PAIR ? tc.m_blk * 2 * BM + BM * static_cast<int>(rank) + row : tc.m_blk * BM * MT + row;
             const bool row_ok = i < P.rows_p;
-            const float fi = row_ok ? __fmul_rn(P.alpha, __ldca(P.sp + (P.sp_mode ? i : 0))) : 0.0f;
+            const float fi = row_ok ? __fmul_rn(P.alpha, load_scale<kPinScales>(P.sp + (P.sp_mode ? i : 0))) : 0.0f;
             const int jbase = tc.n_blk * P.bn;
             // every column scale of the tile reaches L1 while its MMAs run:
             // read window by window during the epilogue, each would
@@ -1365,7 +1385,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                 c_hi = c_lo + C::kDrainFirst;
             }
             ScaleWindows sw;
-            sw.init(P, jbase + c_lo, lane, c_hi - c_lo);
+            sw.init(P, jbase + c_lo, lane, c_hi - c_lo, kPinScales);
             // the whole warp takes the same branch (tcgen05.ld is warp-collective)
             const bool got = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, wlim);
             if (!__all_sync(0xFFFFFFFFu, got)) {
@@ -1504,7 +1524,7 @@ __global__ void __launch_bounds__(Cfg<MT, SP, BNC, KC, MX, PAIR>::kThreads, 1)
                                                                                 sw, tmC, c_lo, c_hi, held);
                 c_lo = acc ? C::kDrainFirst : 0;
                 c_hi = acc ? c_end : c_end - C::kDrainFirst;
-                sw.init(P, jbase + c_lo, lane, c_hi - c_lo);
+                sw.init(P, jbase + c_lo, lane, c_hi - c_lo, kPinScales);
             }
             // (block-scaled pairs are never transposed: build_plan_tiles)
             if (!P.trans_out || (PAIR && MX)) {
@@ -2267,9 +2287,11 @@ TileChoice choose(const Job* jobs, const int* bns, int n, int max_ctas, const Ti
 // of A and gains less: up to K 2048 as much as 11 % slower, 3072 and 4096 level
 // and 1 to 7 % faster for 192 (1000 x 5120 x 4096 20.9 -> 19.7; transposed
 // outputs 5 % slower to 5 % faster, so not there), from 6144 on 2 %; faster at
-// every K where the width leaves out a tenth of the columns, padding (8192 x
-// 512 x 1024: 10.7 -> 9.9 us), or where unaligned output rows make the epilogue
-// the longest part of a tile (1536 x 3001 x 1024: 22.0 -> 15.6).
+// every K where the width leaves a twelfth of the columns out, padding (8192 x
+// 512 x 1024: 10.7 -> 9.9 us; 4096 x 1024 x 1024 transposed 11.6 -> 10.5).
+// Either kind is faster at every K where unaligned output rows make the
+// epilogue the longest part of a tile (2:4 1536 x 3001 x 1024: 22.0 -> 15.6,
+// dense 4096 x 1029 x 1024 18.5 -> 15.6; 2048 x 3001 3 % slower).
 int pair_width(const Job& j, int widest, int pairs)
 {
     const bool sparse = j.E != nullptr;
@@ -2285,10 +2307,12 @@ int pair_width(const Job& j, int widest, int pairs)
         return kLaunch + static_cast<double>(waves * k_blocks) * block;
     };
     const auto measured_faster = [&](int w) {
+        if (unaligned)
+            return true;
         if (!sparse)
             return k_blocks >= 16;
-        return k_blocks >= 48 || (k_blocks >= 24 && w >= 192 && !j.trans_out) || unaligned ||
-               10 * columns(w) <= 9 * columns(widest);
+        return k_blocks >= 48 || (k_blocks >= 24 && w >= 192 && !j.trans_out) ||
+               100 * columns(w) <= 92 * columns(widest);
     };
     int best = widest;
     double best_cost = 0.95 * cost(widest);
