@@ -171,7 +171,8 @@ int fp8_quantize_e4m3_rows_grouped(const fp8_quant_job *jobs, int num_jobs, fp8_
  * B [N, K] (ldb) codes as in gemm_fp8_dense (16-byte aligned, strides
  * multiples of 16); a_scales / b_scales: the tiled layout of A's and B's
  * scales (16-byte aligned).  K % 32 == 0 (FP8_ERR_SHAPE otherwise).  C, ldc,
- * out_dtype, formats and stream as gemm_fp8_dense_fmt.  Needs no workspace.
+ * out_dtype, formats and stream as gemm_fp8_dense_fmt.  Needs no workspace
+ * (slices of skinny products along K add up within thread-block clusters).
  * ------------------------------------------------------------------------- */
 size_t fp8_mx_scale_tiled_bytes(int64_t rows, int64_t cols);
 
@@ -413,7 +414,7 @@ int gemm_fp8_grouped_ex(const fp8_gemm_problem *problems, int num_problems, int 
  * CTA of a two-CTA cluster loads 128 rows of A and 128 rows of B and holds
  * its half of the accumulator; 2:4 launches take 256 x 224 pair tiles,
  * each CTA loading the kept codes and metadata of its 128 rows of A and
- * 112 rows of B; dense launches whose N tiles are 256 wide and 2:4 launches
+ * 112 rows of B; with mt 0 a launch of one problem may take narrower ones; dense launches whose N tiles are 256 wide and 2:4 launches
  * whose N tiles are at least 224 wide, otherwise as 0), 0 = chosen per
  * launch (256-row tiles when every problem fills them with N tiles >= 128
  * wide and those tiles number at least half the SMs, or, for CTA pairs
@@ -464,7 +465,7 @@ int gemm_fp8_dense_plan(int64_t M, int64_t N, int64_t K, int out_dtype, fp8_gemm
 int gemm_fp8_mx_plan(int64_t M, int64_t N, int64_t K, int out_dtype, fp8_gemm_plan_info *info);
 
 /* How gemm_fp8_sparse24 would run an M x N x K 2:4 problem now: mt 3 (CTA
- * pairs, 256 x 224 tiles, two accumulators per CTA), mt 2 (256-row tiles of
+ * pairs, 256 x 224 tiles or narrower, two accumulators per CTA), mt 2 (256-row tiles of
  * one CTA, N <= 224) or mt 1 (128-row tiles).  A is always the sparse side
  * (swapped = 0).  FP8_ERR_SHAPE unless K % 128 == 0.  Paper: section 6 (2:4
  * sparse GEMM against dense on the same operands). */

@@ -48,8 +48,9 @@ __device__ __forceinline__ uint32_t byte_sign_mask(uint32_t v)
 // least two of its three comparisons, a majority, which is one three-input
 // logic instruction for all four groups.  The same pair as select_group's
 // tournament in about 12 instructions a group (the two-groups-per-register
-// tournament this replaced took about 30, and the ALU pipe was the limit of
-// prune24_compress: 77 % busy at 8192 x 8192).  Returns the four index
+// tournament this replaced took about 30, and they were what limited
+// prune24_compress: 23.3 -> 17.3 us at 8192 x 8192 with rows taken as one
+// run).  Returns the four index
 // nibbles (group g in bits 4g .. 4g + 3) and the kept codes of groups 0, 1
 // and 2, 3 in v01 and v23 (lower index first).
 __device__ __forceinline__ uint32_t select_groups4(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,

@@ -130,8 +130,8 @@ __device__ __forceinline__ void scale_from_amax(uint32_t amax_bits, float& s, fl
 // threads per row that read it twice: 16384 x 4096 58.0 -> 49.2 us (6.8
 // TB/s), 16384 x 14336 183 -> 165 us (7.1 TB/s), 16384 x 512 28.5 -> 8.5 us,
 // 16 x 14336 3.4 -> 2.5 us.  Fused with 2:4 compression: 14336 x 4096 64.7
-// -> 50.2 us (6.6 TB/s), 16384 x 16384 250 -> 216 us (its ALU pipe was 68 %
-// busy: the four-group selection took half of that away).  1024 x 32768 47.7
+// -> 50.2 us (6.6 TB/s), 16384 x 16384 250 -> 216 us (the
+// four-group selection takes less than half of the instructions).  1024 x 32768 47.7
 // -> 29.8 us.
 constexpr int kRowBlock = 256;            // threads of a block where TPR is smaller
 constexpr int kRowMaxCols = 32768;        // longest row held in registers

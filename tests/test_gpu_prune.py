@@ -142,3 +142,25 @@ def test_expand_to_any_byte(orc, M, K):
         gb.prune24_decompress(v, m, K, out=out)
         assert np.array_equal(out.cpu().numpy(), want)
         assert bool((buf[:off] == 0xA5).all()) and bool((buf[-5:] == 0xA5).all())
+
+
+def test_expand_any_index_nibble_by_value():
+    """Every metadata byte against the rule itself, on the vector path, the
+    piece path and the group path: code 0 of a group at index nibble & 3,
+    code 1 at nibble >> 2, both OR-ed where the indices agree."""
+    import paper_2602_10262_gb300 as gb
+    M, K = 8, 1024                                        # 256 metadata bytes in each two rows
+    g = np.random.default_rng(4)
+    vals = g.integers(0, 256, (M, K // 2), dtype=np.uint8)
+    meta = np.stack([g.permutation(256).astype(np.uint8) for _ in range(M // 2)]).reshape(M, K // 8)
+    nib = np.stack([meta & 15, meta >> 4], -1).reshape(M, K // 4)
+    want = np.zeros((M, K // 4, 4), np.uint8)
+    r, c = np.indices(nib.shape)
+    pair = vals.reshape(M, K // 4, 2)
+    want[r, c, nib & 3] |= pair[..., 0]
+    want[r, c, nib >> 2] |= pair[..., 1]
+    v, m = torch.from_numpy(vals).cuda(), torch.from_numpy(meta).cuda()
+    for off in (0, 4, 1):
+        out = torch.zeros(M * K + off, dtype=torch.uint8, device="cuda")[off:].view(M, K)
+        gb.prune24_decompress(v, m, K, out=out)
+        assert np.array_equal(out.cpu().numpy(), want.reshape(M, K))
